@@ -42,7 +42,7 @@ struct AdjArgs {
 __device__ __forceinline__ int wp(int i, int n) { return i >= n ? i - n : (i < 0 ? i + n : i); }
 
 // the prescribed velocity at node (x, y) from the velocity tables of type CF (the forward step's), as the
-// forward step forms it: X Y T, two rounded products
+// forward step forms it: X ((Y/12) T), times 12
 template <typename CF>
 __device__ __forceinline__ void vel_at(const InstDev& I, const CF* tabs, const AdjArgs& a, int x, int y, CF T, CF& ux,
                                        CF& uy)
@@ -51,8 +51,8 @@ __device__ __forceinline__ void vel_at(const InstDev& I, const CF* tabs, const A
     const CF* tX2 = tX1 + a.pitch;
     const CF* tY1 = tX2 + a.pitch;
     const CF* tY2 = tY1 + a.ylen;
-    ux = node_u(tX1[x + GC], tY1[y + GR], T);
-    uy = node_u(tX2[x + GC], tY2[y + GR], T);
+    ux = op_mul(CF(12), node_u(tX1[x + GC], op_mul(tY1[y + GR], T)));
+    uy = op_mul(CF(12), node_u(tX2[x + GC], op_mul(tY2[y + GR], T)));
 }
 
 template <typename C> __device__ __forceinline__ C d2f(C phi, C beta, C phiA, C phiB)

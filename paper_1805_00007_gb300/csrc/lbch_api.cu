@@ -22,6 +22,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -463,20 +464,17 @@ void derive(const lbch_params& p, InstDev& d)
     f.K = (float)c.K; f.phiA = (float)c.phiA; f.phiB = (float)c.phiB;
     f.itau = (float)c.itau; f.omt = (float)c.omt; f.src = (float)c.src;
     f.cF1 = (float)c.cF1; f.cmu = (float)c.cmu;
-    // the collision's per-class coefficients, each one product rounded in the kernel's arithmetic type
-    // (the same rounding as forming them at a node would give)
-    auto coll = [](auto& k) {
-        using T = decltype(k.itau);
-        const T w1 = T(1) / T(9), w5 = T(1) / T(36);
-        k.k1a = w1 * k.itau;
-        k.k1d = w5 * k.itau;
-        k.k2a = T(3) * k.k1a;
-        k.k2d = T(3) * k.k1d;
-        k.k3a = (T(3) * w1) * k.src;
-        k.k3d = (T(3) * w5) * k.src;
+    // the products the per-node arithmetic takes (lbch_kernels.cuh), formed in double and rounded once
+    const double k3 = c.src / 12.0;  // 3 w_5 src
+    const double k[9] = {4.0 * c.beta, -2.0 * c.beta * (p.phiA + p.phiB), c.itau / 36.0 * c.eta,
+                         -144.0 * c.a / c.src, -144.0 * c.b / c.src, k3 * c.K / 12.0, k3, c.cF1 / k3, c.cmu / 12.0};
+    auto products = [&](auto& o) {
+        using T = std::remove_reference_t<decltype(o.beta)>;
+        o.b4 = (T)k[0]; o.b2s = (T)k[1]; o.kM = (T)k[2]; o.ra = (T)k[3]; o.rb = (T)k[4];
+        o.Kd = (T)k[5]; o.k3 = (T)k[6]; o.hF = (T)k[7]; o.hG = (T)k[8];
     };
-    coll(c);
-    coll(f);
+    products(c);
+    products(f);
     d.Tper = p.Tper;
     d.walls = p.walls; d.model = p.model; d.vel = p.vel;
 }
@@ -484,7 +482,8 @@ void derive(const lbch_params& p, InstDev& d)
 // The prescribed flows are separable: ux = X1(x) Y1(y) T(t), uy = X2(x) Y2(y) T(t).  The tables are
 // indexed like the stored arrays: X1, X2 by stored column (domain x = column - GC, periodic images in
 // the ghost columns), Y1, Y2 by row of the instance's stored band (domain y = row - GR; periodic or
-// mirror images in the ghost rows, matching the stored phi), then Y1, Y2 at the walls y = -1/2, ny - 1/2.
+// mirror images in the ghost rows, matching the stored phi) and divided by 12 (the kernels work with u/12), then
+// Y1, Y2 themselves at the walls y = -1/2, ny - 1/2.
 // A slab of a larger periodic grid (lb_ch_init_slab): the handle holds global rows y0 .. y0 + ny - 1.
 struct SlabSpec {
     int y0;   // first global row of the slab
@@ -537,6 +536,8 @@ void velocity_tables(const lbch_params& p, int pitch, int ylen, std::vector<doub
         if (slab) yy = (((slab->y0 + y) % p.ny) + p.ny) % p.ny;  // the global row a slab's row stands for
         else yy = p.walls ? (y < 0 ? -1 - y : (y >= p.ny ? 2 * p.ny - 1 - y : y)) : ((y % p.ny) + p.ny) % p.ny;
         Y((double)yy, Y1[k], Y2[k]);
+        Y1[k] /= 12.0;
+        Y2[k] /= 12.0;
     }
     Y(-0.5, W[0], W[2]);
     Y((double)p.ny - 0.5, W[1], W[3]);

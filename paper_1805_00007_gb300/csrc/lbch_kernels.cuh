@@ -48,9 +48,14 @@ struct Consts {
     C beta, kappa, eta, a, b, K, phiA, phiB;
     C itau, omt, src;  // 1/tau, 1 - 1/tau, 1 - 1/(2 tau)
     C cF1, cmu;        // Model III: 2 tau - 1 + 3K and 3 c_s^2 eta K, the coefficients of d_t F1 and d_t grad mu
-    // the collision's coefficients per direction class (axis a, diagonal d), each one rounded product:
-    // w/tau, 3 (w/tau), (3 w)(1 - 1/(2 tau)), formed once at set-up rather than at every node
-    C k1a, k1d, k2a, k2d, k3a, k3d;
+    // Products of the above as the step's per-node arithmetic takes them (formed in double at set-up and rounded
+    // once), so that no node multiplies by a constant that another constant could carry:
+    C b4, b2s;         // 4 beta and -2 beta (phiA + phiB): f'(phi) = (phi - phiA)(phi - phiB)(b4 phi + b2s)
+    C kM;              // (w_5 / tau) eta
+    C ra, rb;          // -144 a / src, -144 b / src: 1/(ra phi + rb) = -(3 w_5 src)/(12 rho)
+    C Kd;              // 3 w_5 src K / 12
+    C k3;              // 3 w_5 src
+    C hF, hG;          // Model III: cF1 / k3 and cmu / 12
 };
 
 // Per-instance parameters, derived constants and layout, resident in device memory.
@@ -60,7 +65,7 @@ struct InstDev {
     int walls, model, vel;
     int ylen;          // length of each Y velocity table: ny rounded up to 16, plus 24 (ghost rows and the
                        // reach of the last tile's slice)
-    int tab;           // offset of the velocity tables: X1, X2 [pitch]; Y1, Y2 [ylen]; W[4]
+    int tab;           // offset of the velocity tables: X1, X2 [pitch]; Y1/12, Y2/12 [ylen]; W[4]
     int slab;          // a slab of a larger periodic grid: its ghost rows hold the neighbouring slabs' rows
                        // (imported between steps), not images of its own rows
     double Tper;
@@ -80,7 +85,8 @@ struct Ctl {
     unsigned int err;   // bit 0: a TMA wait timed out
 };
 
-// Time factor of the prescribed flows: u(x, y, t) = (X1(x) Y1(y), X2(x) Y2(y)) T(t).
+// Time factor of the prescribed flows: u(x, y, t) = (X1(x) Y1(y), X2(x) Y2(y)) T(t).  The tables hold Y1/12 and
+// Y2/12, and the kernels work with u/12 (node_u), the scale at which the stencils of div(phi u) take it.
 __host__ __device__ inline double vel_t(int vel, double Tper, long long n)
 {
     const double pi = 3.14159265358979323846;
@@ -138,129 +144,193 @@ __device__ __forceinline__ int mirror(int j, int n)
 }
 
 // ------------------------------------------------------------------------------------------ per-node arithmetic
-// Used by both forms of the step kernel (tiles in shared memory; row sweeps in registers), so that every
-// quantity is evaluated by the same operations in both.  Every product is an explicit rounded multiply
-// or an explicit fused multiply-add: the compiler's own contraction of a*b + c depends on how often a
-// product is reused, which differs between the two forms, and would change the last bits.
+// Used by every form of the step kernel (tiles in shared memory; row sweeps in registers; two steps per
+// launch), so that every quantity is evaluated by the same operations in all of them.  Every product is an
+// explicit rounded multiply or an explicit fused multiply-add: the compiler's own contraction of a*b + c
+// depends on how often a product is reused, which differs between the forms, and would change the last bits.
+//
+// The isotropic nine-point stencils are products of one-dimensional ones, and are evaluated as such: first a few
+// values per column from the nodes below, at and above a row, then their combination along the row.  A form
+// that holds the column values (the row sweep) forms them once per node, and every constant that another can
+// carry is folded into it at set-up.  A node's update at tau_g = 1, Model II, takes 87 operations this way
+// (streaming and the float-float sum included) where the nine-point forms direction by direction took 149.  The
+// FP64 kernels, which the FP64 pipe bounds, and the row sweeps, which instruction issue bounds, gained most
+// (us per step before -> after: FP64 500^2 row sweep 147 -> 94, FP64 256^2 two-step kernel 30.6 -> 23.8, float
+// 3001 x 1999 row sweep 65.7 -> 53.3, half storage with the populations at 4096^2 267 -> 219; float with the
+// populations, near its HBM bound, 297 -> 295), with the same distance from the 64-bit result.
 __device__ __forceinline__ float op_mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double op_mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float op_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double op_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// d/dphi of beta (phi - phiA)^2 (phi - phiB)^2 (Eq. bulk)
+// Reciprocal for the force: the hardware's approximation (about 23 bits in float, 20 in double) refined once,
+// in float by r + r (1 - v r), in double by the third-order r + r (e + e^2), e = 1 - v r (2^-20 -> 2^-60).
+__device__ __forceinline__ float node_rcp(float v)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return op_fma(r, op_fma(-v, r, 1.0f), r);
+}
+__device__ __forceinline__ double node_rcp(double v)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+    const double e = op_fma(-v, r, 1.0);
+    return op_fma(r, op_fma(e, e, e), r);
+}
+
+// d/dphi of beta (phi - phiA)^2 (phi - phiB)^2 (Eq. bulk), direction by direction (the coupled flow)
 template <typename C> __device__ __forceinline__ C node_dfdphi(C phi, C beta, C phiA, C phiB)
 {
     const C s = op_fma(C(2), phi, -phiA) - phiB;
     return op_mul(op_mul(op_mul(op_mul(C(2), beta), phi - phiA), phi - phiB), s);
 }
 
-// Eq. mu: mu = f'(phi) - kappa lap phi, with the isotropic nine-point Laplacian
-// lap psi = sum_k 2 w_k (psi(x + c_k) - psi(x)) / c_s^2.
-template <typename C>
-__device__ __forceinline__ C node_mu(C ce, C pE, C pW, C pN, C pS, C pNE, C pNW, C pSE, C pSW, C beta, C kappa,
-                                     C phiA, C phiB)
+// Column values of phi for the Laplacian: dl = the second difference along y, and z = phi + dl/6.  The isotropic
+// Laplacian sum_k 2 w_k (psi(x + c_k) - psi(x)) / c_s^2 is dl + (z(E) - 2 z + z(W)).
+template <typename C> __device__ __forceinline__ C node_z(C pS, C ce, C pN, C& dl)
 {
-    const C ax = (pE + pW) + (pN + pS);
-    const C dg = (pNE + pNW) + (pSE + pSW);
-    const C lap = op_fma(C(2) / C(3), op_fma(C(-4), ce, ax), op_mul(C(1) / C(6), op_fma(C(-4), ce, dg)));
-    return op_fma(-kappa, lap, node_dfdphi(ce, beta, phiA, phiB));
+    dl = op_fma(C(-2), ce, pN + pS);
+    return op_fma(C(1) / C(6), dl, ce);
 }
 
-// D = div(phi u) = sum_k w_k c_k . (phi u)(x + c_k) / c_s^2 for the separable flow u = (X1 Y1, X2 Y2) T:
-// x*m / x*c / x*p are the X tables at column offsets -1 / 0 / +1, y*m / y*c / y*p the Y tables at row
-// offsets -1 / 0 / +1.  D is linear in u, so the time factor T multiplies once at the end.
-template <typename C>
-__device__ __forceinline__ C node_div(C pE, C pW, C pN, C pS, C pNE, C pNW, C pSE, C pSW, C x1m, C x1p, C x2m, C x2c,
-                                      C x2p, C y1m, C y1c, C y1p, C y2m, C y2p, C T)
+// Eq. mu: mu = f'(phi) - kappa lap phi, with f' of Eq. bulk in its factors
+template <typename C> __device__ __forceinline__ C node_mu(C ce, C dl, C z, C zE, C zW, const Consts<C>& K0)
 {
-    // axis neighbours: (phi ux)(E) - (phi ux)(W) + (phi uy)(N) - (phi uy)(S)
-    const C ax1 = op_fma(pE, op_mul(x1p, y1c), -op_mul(pW, op_mul(x1m, y1c)))
-                + op_fma(pN, op_mul(x2c, y2p), -op_mul(pS, op_mul(x2c, y2m)));
-    // diagonal neighbours: c_k . (phi u)(x + c_k) for NE, NW, SW, SE
-    const C bNE = op_fma(x1p, y1p, op_mul(x2p, y2p));
-    const C bNW = op_fma(x2m, y2p, -op_mul(x1m, y1p));
-    const C bSW = op_fma(x1m, y1m, op_mul(x2m, y2m));
-    const C bSE = op_fma(x1p, y1m, -op_mul(x2p, y2m));
-    const C dg1 = op_fma(pSE, bSE, op_fma(-pSW, bSW, op_fma(pNW, bNW, op_mul(pNE, bNE))));
-    return op_mul(op_fma(C(1) / C(3), ax1, op_mul(C(1) / C(12), dg1)), T);
+    const C lap = dl + op_fma(C(-2), z, zE + zW);
+    const C f1 = op_mul(op_mul(ce - K0.phiA, ce - K0.phiB), op_fma(K0.b4, ce, K0.b2s));
+    return op_fma(-K0.kappa, lap, f1);
 }
 
-// Isotropic gradient grad psi = sum_k w_k c_k psi(x + c_k) / c_s^2.
+// Column values of the flux phi u for D = div(phi u) = sum_k w_k c_k . (phi u)(x + c_k) / c_s^2 in the separable flow
+// u = (X1 Y1, X2 Y2) T: with y1 = Y1 T/12, y2 = Y2 T/12 of the rows below (S), at (y14 = 4 y1) and above (N), the
+// column's share in D of the node to its west is E, to its east W, and of its own node 4 d.
+template <typename C>
+__device__ __forceinline__ C node_flux(C pS, C ce, C pN, C X1, C X2, C y1S, C y14, C y1N, C y2S, C y2N, C& E, C& W)
+{
+    const C t = op_fma(y1N, pN, op_fma(y1S, pS, op_mul(y14, ce)));
+    const C d = op_mul(X2, op_fma(y2N, pN, -op_mul(y2S, pS)));
+    E = op_fma(X1, t, d);
+    W = op_fma(-X1, t, d);
+    return d;
+}
+// ... its own node's alone
+template <typename C> __device__ __forceinline__ C node_flux_d(C pS, C pN, C X2, C y2S, C y2N)
+{
+    return op_mul(X2, op_fma(y2N, pN, -op_mul(y2S, pS)));
+}
+// D from the node's own d, the E of the column to its east and the W of the column to its west
+template <typename C> __device__ __forceinline__ C node_div(C d, C E, C W) { return op_fma(C(4), d, E + W); }
+
+// Column values of a field for the isotropic gradient sum_k w_k c_k psi(x + c_k) / c_s^2 = (gx, gy)/12:
+// w = psi(S) + 4 psi + psi(N) and d = psi(N) - psi(S); gx = w(E) - w(W), gy = d(E) + 4 d + d(W).
+template <typename C> __device__ __forceinline__ C node_w(C s, C c, C n) { return op_fma(C(4), c, n + s); }
+template <typename C> __device__ __forceinline__ C node_gy(C dW, C d, C dE) { return op_fma(C(4), d, dE + dW); }
+
+// The same from the nine values of a node's neighbourhood (the forms that hold fields in shared memory).
+template <typename C>
+__device__ __forceinline__ C mu9(C ce, C pE, C pW, C pN, C pS, C pNE, C pNW, C pSE, C pSW, const Consts<C>& K0)
+{
+    C dl, dE, dW;
+    const C z = node_z(pS, ce, pN, dl), zE = node_z(pSE, pE, pNE, dE), zW = node_z(pSW, pW, pNW, dW);
+    return node_mu(ce, dl, z, zE, zW, K0);
+}
+// x1*, x2*: the X tables at the columns W, (C), E; y1*, y2*: the Y tables (times T) at the rows S, (C), N
+template <typename C>
+__device__ __forceinline__ C div9(C pE, C pW, C pN, C pS, C pNE, C pNW, C pSE, C pSW, C x1W, C x1E, C x2W, C x2C,
+                                  C x2E, C y1S, C y1C, C y1N, C y2S, C y2N)
+{
+    const C y14 = op_mul(C(4), y1C);
+    C EE, WE, EW, WW;
+    node_flux(pSE, pE, pNE, x1E, x2E, y1S, y14, y1N, y2S, y2N, EE, WE);
+    node_flux(pSW, pW, pNW, x1W, x2W, y1S, y14, y1N, y2S, y2N, EW, WW);
+    return node_div(node_flux_d(pS, pN, x2C, y2S, y2N), EE, WW);
+}
 template <typename C>
 __device__ __forceinline__ void grad9(C E, C W, C N, C S, C NE, C NW, C SE, C SW, C& gx, C& gy)
 {
-    gx = op_fma(C(1) / C(3), E - W, op_mul(C(1) / C(12), (NE - NW) + (SE - SW)));
-    gy = op_fma(C(1) / C(3), N - S, op_mul(C(1) / C(12), (NE + NW) - (SE + SW)));
+    gx = node_w(SE, E, NE) - node_w(SW, W, NW);
+    gy = node_gy(NW - SW, N - S, NE - SE);
 }
 
-// The force: F1 = (phi / rho)(-phi grad mu) with rho = a phi + b (Eq. liangFi, with grad p = 0), plus
-// F2 = 3 c_s^2 K grad(div(phi u)) for Model II (Eq. mark3).
+// The prescribed velocity over 12 at a node, X(x) y(y) with y = (Y/12) T.
+template <typename C> __device__ __forceinline__ C node_u(C X, C y) { return op_mul(X, y); }
+// ... and at a wall (the tables' W entries hold Y itself there)
+template <typename C> __device__ __forceinline__ C wall_u(C X, C W, C T) { return op_mul(X, op_mul(W, T)); }
+
+// 1/tau phi u, the momentum part of g_eq in the scale of the diagonal directions: 3 w_5 / tau phi u = 1/tau phi (u/12)
 template <typename C>
-__device__ __forceinline__ void node_force(C ph, C gmx, C gmy, C gDx, C gDy, bool model2, C ra, C rb, C K, C& Fx,
-                                           C& Fy)
+__device__ __forceinline__ void node_flow(C ph, C ux, C uy, const Consts<C>& K0, C& Px, C& Py)
 {
-    const C fct = op_mul(op_mul(-ph, ph), rcp<C>(op_fma(ra, ph, rb)));
-    Fx = op_mul(fct, gmx);
-    Fy = op_mul(fct, gmy);
-    if (model2) {
-        Fx = op_fma(K, gDx, Fx);
-        Fy = op_fma(K, gDy, Fy);
-    }
+    const C pk = op_mul(K0.itau, ph);
+    Px = op_mul(pk, ux);
+    Py = op_mul(pk, uy);
+}
+
+// The part of g_eq / tau + (1 - 1/(2 tau)) S odd in c_i, in the scale of the diagonal directions: J = 3 w_5 (phi u/tau +
+// (1 - 1/(2 tau)) F).  F1 = (phi / rho)(-phi grad mu) with rho = a phi + b (Eq. liangFi, with grad p = 0), plus
+// F2 = 3 c_s^2 K grad(div(phi u)) for Model II (Eq. mark3).  gm, gD: 12 grad mu, 12 grad D.
+template <typename C>
+__device__ __forceinline__ void node_force(C ph, C gmx, C gmy, C gDx, C gDy, C Px, C Py, bool model2,
+                                           const Consts<C>& K0, C& Jx, C& Jy)
+{
+    const C fct = op_mul(op_mul(ph, ph), node_rcp(op_fma(K0.ra, ph, K0.rb)));
+    Jx = op_fma(fct, gmx, model2 ? op_fma(K0.Kd, gDx, Px) : Px);
+    Jy = op_fma(fct, gmy, model2 ? op_fma(K0.Kd, gDy, Py) : Py);
 }
 
 // Model III: the complete diffusive-scale force of Eq. F2-1, with the time derivatives on the convective
 // scale replaced by backward differences over one step (Remarks I, II).  H = cF1 F1 + cmu grad mu is the
 // part under the time derivative; F = F1 + (H - Hprev) + 3 c_s^2 K grad D.  Hprev = H at the first step.
 template <typename C>
-__device__ __forceinline__ void node_force_full(C ph, C gmx, C gmy, C gDx, C gDy, C Hpx, C Hpy, bool first, C ra, C rb,
-                                                C K, C cF1, C cmu, C& Fx, C& Fy, C& Hx, C& Hy)
+__device__ __forceinline__ void node_force_full(C ph, C gmx, C gmy, C gDx, C gDy, C Hpx, C Hpy, bool first, C Px, C Py,
+                                                const Consts<C>& K0, C& Jx, C& Jy, C& Hx, C& Hy)
 {
-    C F1x, F1y;
-    node_force(ph, gmx, gmy, C(0), C(0), false, ra, rb, K, F1x, F1y);
-    Hx = op_fma(cF1, F1x, op_mul(cmu, gmx));
-    Hy = op_fma(cF1, F1y, op_mul(cmu, gmy));
+    const C fct = op_mul(op_mul(ph, ph), node_rcp(op_fma(K0.ra, ph, K0.rb)));
+    Hx = op_fma(K0.hF, op_mul(fct, gmx), op_mul(K0.hG, gmx));
+    Hy = op_fma(K0.hF, op_mul(fct, gmy), op_mul(K0.hG, gmy));
     const C dHx = first ? C(0) : Hx - Hpx, dHy = first ? C(0) : Hy - Hpy;
-    Fx = op_fma(K, gDx, F1x + dHx);
-    Fy = op_fma(K, gDy, F1y + dHy);
+    Jx = op_fma(fct, gmx, op_fma(K0.k3, dHx, op_fma(K0.Kd, gDx, Px)));
+    Jy = op_fma(fct, gmy, op_fma(K0.k3, dHy, op_fma(K0.Kd, gDy, Py)));
 }
-
-// The prescribed velocity X(x) Y(y) T at a node.
-template <typename C> __device__ __forceinline__ C node_u(C X, C Y, C T) { return op_mul(op_mul(X, Y), T); }
 
 // Eq. LB as g* = (1 - 1/tau) g + g_eq / tau + (1 - 1/(2 tau)) S, with Eq. geq and the source
-// S_i = w_i c_i . F / c_s^2 (Eq. liangFi), split into the parts even and odd in c_i.  With kShift the
-// rest population is carried as g_0 - phi.  With TAU1 (tau = 1) the populations g are not read.  PRE:
-// take the per-class coefficients precomputed in K0, else form them here (the same rounded products, so
-// the same bits; which is faster depends on the kernel's register budget).
-template <typename C, bool TAU1, bool kShift, bool PRE = true>
-__device__ __forceinline__ void collide9(C ph, C mu, C Fx, C Fy, C ux, C uy, const C* g, const Consts<C>& K0, C* post)
+// S_i = w_i c_i . F / c_s^2 (Eq. liangFi), split into the parts even and odd in c_i (J, node_force).  ux, uy:
+// u/12; Px, Py: node_flow.  The rest population leaves out phi/tau (it is carried as g_0 - phi in the float
+// paths; rest_add puts it back in double).  Everything is formed in the scale of the diagonal directions
+// (w_5 = w_1/4); q = 0: the full value.  With QUARTER (tau_g = 1, where the populations are not read) the axis
+// directions 1..4 are returned in that scale, a quarter of g*, for stream_sum_q to multiply in its sums;
+// otherwise every g* is returned in full, with the same bits (a multiplication by 4 is exact).
+template <typename C, bool QUARTER>
+__device__ __forceinline__ void collide9(C mu, C ux, C uy, C Px, C Py, C Jx, C Jy, const C* g, const Consts<C>& K0, C* post)
 {
-    const C itau = K0.itau, omt = K0.omt;
-    // per direction class (axis, diagonal): w/tau, 3 w/tau, 3 w (1 - 1/(2 tau))
-    const C k1a = PRE ? K0.k1a : op_mul(wq<C>(1), itau), k1d = PRE ? K0.k1d : op_mul(wq<C>(5), itau);
-    const C k2a = PRE ? K0.k2a : op_mul(C(3), k1a), k2d = PRE ? K0.k2d : op_mul(C(3), k1d);
-    const C k3a = PRE ? K0.k3a : op_mul(C(3) * wq<C>(1), K0.src), k3d = PRE ? K0.k3d : op_mul(C(3) * wq<C>(5), K0.src);
-    const C emu = op_mul(K0.eta, mu);
-    const C phuu = op_mul(ph, op_fma(ux, ux, op_mul(uy, uy)));
-    const C even = op_fma(C(-1.5), phuu, emu);
-    const C ph45 = op_mul(C(4.5), ph);
-    C g0eq = op_fma(wq<C>(0) - C(1), emu, op_mul(-wq<C>(0) * C(1.5), phuu));
-    if (!kShift) g0eq = ph + g0eq;
-    post[0] = TAU1 ? g0eq : op_fma(omt, g[0], op_mul(itau, g0eq));
+    const C M = op_mul(K0.kM, mu);
+    const C tx = op_mul(Px, ux), ty = op_mul(Py, uy), r = op_mul(Px, uy);
+    const C s = tx + ty;
+    const C e = op_fma(C(-6), s, M), Ad = op_fma(C(12), s, M);
     // pairs (q, opp q): (1,3) c=(1,0); (2,4) c=(0,1); (5,7) c=(1,1); (6,8) c=(-1,1)
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        const int q = (k == 0) ? 1 : (k == 1) ? 2 : (k == 2) ? 5 : 6;
-        const int o = opp(q);
-        const C cu = (k == 0) ? ux : (k == 1) ? uy : (k == 2) ? ux + uy : uy - ux;
-        const C cF = (k == 0) ? Fx : (k == 1) ? Fy : (k == 2) ? Fx + Fy : Fy - Fx;
-        const C k1 = (q < 5) ? k1a : k1d, k2 = (q < 5) ? k2a : k2d, k3 = (q < 5) ? k3a : k3d;
-        const C A = op_mul(k1, op_fma(op_mul(ph45, cu), cu, even));
-        const C B = op_fma(k2, op_mul(ph, cu), op_mul(k3, cF));
-        post[q] = TAU1 ? A + B : op_fma(omt, g[q], A + B);
-        post[o] = TAU1 ? A - B : op_fma(omt, g[o], A - B);
+    const C A1 = op_fma(C(18), tx, e), A2 = op_fma(C(18), ty, e);
+    const C A5 = op_fma(C(36), r, Ad), A6 = op_fma(C(-36), r, Ad);
+    const C J5 = Jx + Jy, J6 = Jy - Jx;
+    const C g0 = op_fma(C(-96), s, op_mul(C(-20), M));
+    if constexpr (QUARTER) {
+        post[0] = g0;
+        post[1] = A1 + Jx; post[3] = A1 - Jx;
+        post[2] = A2 + Jy; post[4] = A2 - Jy;
+        post[5] = A5 + J5; post[7] = A5 - J5;
+        post[6] = A6 + J6; post[8] = A6 - J6;
+    } else {
+        const C omt = K0.omt;
+        post[0] = op_fma(omt, g[0], g0);
+        post[1] = op_fma(omt, g[1], op_mul(C(4), A1 + Jx)); post[3] = op_fma(omt, g[3], op_mul(C(4), A1 - Jx));
+        post[2] = op_fma(omt, g[2], op_mul(C(4), A2 + Jy)); post[4] = op_fma(omt, g[4], op_mul(C(4), A2 - Jy));
+        post[5] = op_fma(omt, g[5], A5 + J5); post[7] = op_fma(omt, g[7], A5 - J5);
+        post[6] = op_fma(omt, g[6], A6 + J6); post[8] = op_fma(omt, g[8], A6 - J6);
     }
 }
+
+// The rest population of the double path from collide9's: phi/tau added
+template <typename C> __device__ __forceinline__ C rest_add(C g0, C ph, const Consts<C>& K0) { return op_fma(K0.itau, ph, g0); }
 
 // Halfway bounce-back at a wall node: g_q arriving from the ghost row is the node's own post-collision
 // g_opp(q) plus the moving-wall term 2 w_q phi (c_q . u_w) / c_s^2.
@@ -279,6 +349,13 @@ template <typename C>
 __device__ __forceinline__ C stream_sum(C v1, C v2, C v3, C v4, C v5, C v6, C v7, C v8)
 {
     return (((v1 + v5) + v8) + (v2 + v4)) + ((v3 + v6) + v7);
+}
+// The same with 1..4 in a quarter (collide9's QUARTER): the same bits, since multiplications by 4 are exact
+template <typename C>
+__device__ __forceinline__ C stream_sum_q(C v1, C v2, C v3, C v4, C v5, C v6, C v7, C v8)
+{
+    const C R = op_fma(C(4), v1, v5) + v8, L = op_fma(C(4), v3, v6) + v7;
+    return op_fma(C(4), v2 + v4, R) + L;
 }
 
 // ------------------------------------------------------------------------------------------ TMA / mbarrier
@@ -462,6 +539,8 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
     constexpr bool kShift = sizeof(C) == 4;   // float arithmetic on g_0 - phi instead of g_0
     constexpr bool kFF = L::FF;
     constexpr int QOFF = kHalf ? 1 : 0;       // stored plane of population q is q - QOFF
+    // at tau_g = 1 the axis populations are staged in a quarter (collide9); not where they round to half
+    constexpr bool kQuarter = TAU1 && !kHalf;
     constexpr int NONE = -0x40000000;
 
     extern __shared__ unsigned char smem_raw[];
@@ -573,15 +652,19 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         const C* tY2 = tY1 + I.ylen;
         const C* tW = tY2 + I.ylen;
 
-        // the velocity-table slices arrived with the boxes: X by box column, Y by box row; the prescribed
-        // velocity at box (row, col) is (X1[col] Y1[row], X2[col] Y2[row]) T
+        // the velocity-table slices arrived with the boxes: X by box column, Y/12 by box row, multiplied here by
+        // the time factor (1 for the flows without one); u/12 at box (row, col) is (X1[col] Y1[row], X2[col] Y2[row])
         const C* sX1 = reinterpret_cast<const C*>(stage(s) + L::OFF_T);
         const C* sX2 = sX1 + BW;
         const C* sY1 = sX2 + BW;
         const C* sY2 = sY1 + L::YT;
+        if (a.need_time) {
+            C* sY = const_cast<C*>(sY1);
+            for (int e = tid; e < 2 * L::YT; e += NT) sY[e] = op_mul(sY[e], T);
+            __syncthreads();
+        }
 
         // 2. mu (Eq. mu) and D = div(phi u) on tile + 2
-        const C beta = K0.beta, kappa = K0.kappa, phiA = K0.phiA, phiB = K0.phiB;
         // (the compact order in every phase: the strided order of for_region measured no faster here, 4.56
         // against 4.55 us per step for 256^2 at tau_g = 0.8 in FP32, 4.30 against 4.23 with half storage)
         for_region<MW, L::MH, MW, NT>([&](int e, int r, int c) {
@@ -589,10 +672,10 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
             C ce = cvt<C>(q[0]);
             C pE = cvt<C>(q[1]), pW = cvt<C>(q[-1]), pN = cvt<C>(q[BW]), pS = cvt<C>(q[-BW]);
             C pNE = cvt<C>(q[BW + 1]), pNW = cvt<C>(q[BW - 1]), pSE = cvt<C>(q[-BW + 1]), pSW = cvt<C>(q[-BW - 1]);
-            s_mu[e] = node_mu(ce, pE, pW, pN, pS, pNE, pNW, pSE, pSW, beta, kappa, phiA, phiB);
+            s_mu[e] = mu9(ce, pE, pW, pN, pS, pNE, pNW, pSE, pSW, K0);
             if (model >= 2)  // the tables at box columns c+1..c+3 and box rows r..r+2
-                s_D[e] = node_div(pE, pW, pN, pS, pNE, pNW, pSE, pSW, sX1[c + 1], sX1[c + 3], sX2[c + 1], sX2[c + 2],
-                                  sX2[c + 3], sY1[r], sY1[r + 1], sY1[r + 2], sY2[r], sY2[r + 2], T);
+                s_D[e] = div9(pE, pW, pN, pS, pNE, pNW, pSE, pSW, sX1[c + 1], sX1[c + 3], sX2[c + 1], sX2[c + 2],
+                              sX2[c + 3], sY1[r], sY1[r + 1], sY1[r + 2], sY2[r], sY2[r + 2]);
         });
         if (walls && (y0 < 2 || y0 + TY + 2 > ny)) {
             // every stencil operand takes at a ghost row the value at the mirror row: mu and D at rows
@@ -613,7 +696,6 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         __syncthreads();
 
         // 3. force, equilibrium, source and collision on tile + 1, written back into the box
-        const C ra = K0.a, rb = K0.b, K = K0.K;
         for_region<GW, L::GH, GW, NT>([&](int e, int r, int c) {
             int gy = y0 - 1 + r;
             if (walls && (gy < 0 || gy >= ny)) return;  // ghost rows: never pulled (bounce-back)
@@ -626,7 +708,9 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
                       s_D[m - MW + 1], s_D[m - MW - 1], gDx, gDy);
             C ph = cvt<C>(pb[(r + 2) * BW + c + 3]);
             C mu = s_mu[m];
-            C Fx, Fy;
+            const C ux = node_u(sX1[c + 3], sY1[r + 2]), uy = node_u(sX2[c + 3], sY2[r + 2]);  // box row r+2, col c+3
+            C Px, Py, Jx, Jy;
+            node_flow(ph, ux, uy, K0, Px, Py);
             if (model == 3) {
                 // H(t - 1) at this node (halo nodes included: its images are stored one deep); H(t) is
                 // stored for the tile's own nodes only
@@ -635,13 +719,12 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
                 const bool first = n == 0;
                 const C Hpx = first ? C(0) : a.H_in[hn], Hpy = first ? C(0) : a.H_in[a.H_plane + hn];
                 C Hx, Hy;
-                node_force_full(ph, gmx, gmy, gDx, gDy, Hpx, Hpy, first, ra, rb, K, K0.cF1, K0.cmu, Fx, Fy, Hx, Hy);
+                node_force_full(ph, gmx, gmy, gDx, gDy, Hpx, Hpy, first, Px, Py, K0, Jx, Jy, Hx, Hy);
                 if (r >= 1 && r <= TY && c >= 1 && c <= TX && gx < nx && gy < ny)
                     store_h(a.H_out, a.H_plane, I.row0, a.pitch, nx, ny, walls, gx, gy, Hx, Hy);
             } else {
-                node_force(ph, gmx, gmy, gDx, gDy, model == 2, ra, rb, K, Fx, Fy);
+                node_force(ph, gmx, gmy, gDx, gDy, Px, Py, model == 2, K0, Jx, Jy);
             }
-            const C ux = node_u(sX1[c + 3], sY1[r + 2], T), uy = node_u(sX2[c + 3], sY2[r + 2], T);  // box row r+2, col c+3
             // the node's populations in the box: row r, plane q - QOFF, column c + 3
             S* gp = gb + (r * NQ) * BW + c + 3;
             C g[9];
@@ -658,7 +741,8 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
                 for (int q = 0; q < 9; q++) g[q] = cvt<C>(gp[q * BW]);
             }
             C post[9];
-            collide9<C, TAU1, kShift>(ph, mu, Fx, Fy, ux, uy, g, K0, post);
+            collide9<C, kQuarter>(mu, ux, uy, Px, Py, Jx, Jy, g, K0, post);
+            if (!kShift) post[0] = rest_add(post[0], ph, K0);
             if (kHalf) {
                 // the rest population takes what the half-rounded moving ones leave of phi (see the row sweep)
                 C rest = C(0);
@@ -688,20 +772,23 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
             if (wallrow) {
                 // populations that would come from a ghost row are bounced back at the node
                 const C ph = cvt<C>(pb[(r + 3) * BW + c + 4]);
+                constexpr C ax = kQuarter ? C(4) : C(1);  // the staged axis populations in full
+                v[1] = op_mul(ax, v[1]); v[2] = op_mul(ax, v[2]); v[3] = op_mul(ax, v[3]); v[4] = op_mul(ax, v[4]);
                 if (gy == 0) {
-                    const C uwx = node_u(tX1[gx + GC], tW[0], T), uwy = node_u(tX2[gx + GC], tW[2], T);
-                    v[2] = bounce<C, 2>(cvt<C>(src[(4 - QOFF) * BW]), ph, uwx, uwy);
+                    const C uwx = wall_u(tX1[gx + GC], tW[0], T), uwy = wall_u(tX2[gx + GC], tW[2], T);
+                    v[2] = bounce<C, 2>(op_mul(ax, cvt<C>(src[(4 - QOFF) * BW])), ph, uwx, uwy);
                     v[5] = bounce<C, 5>(cvt<C>(src[(7 - QOFF) * BW]), ph, uwx, uwy);
                     v[6] = bounce<C, 6>(cvt<C>(src[(8 - QOFF) * BW]), ph, uwx, uwy);
                 }
                 if (gy == ny - 1) {
-                    const C uwx = node_u(tX1[gx + GC], tW[1], T), uwy = node_u(tX2[gx + GC], tW[3], T);
-                    v[4] = bounce<C, 4>(cvt<C>(src[(2 - QOFF) * BW]), ph, uwx, uwy);
+                    const C uwx = wall_u(tX1[gx + GC], tW[1], T), uwy = wall_u(tX2[gx + GC], tW[3], T);
+                    v[4] = bounce<C, 4>(op_mul(ax, cvt<C>(src[(2 - QOFF) * BW])), ph, uwx, uwy);
                     v[7] = bounce<C, 7>(cvt<C>(src[(5 - QOFF) * BW]), ph, uwx, uwy);
                     v[8] = bounce<C, 8>(cvt<C>(src[(6 - QOFF) * BW]), ph, uwx, uwy);
                 }
             }
-            const C sumq = stream_sum(v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8]);
+            const C sumq = kQuarter && !wallrow ? stream_sum_q(v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8])
+                                                : stream_sum(v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8]);
             P hi;
             float lo = 0.0f;
             if (kFF) {
@@ -812,7 +899,7 @@ __global__ void init_kernel(const InstDev* inst, int n_inst, const double* tabs,
     const double* tY1 = tX2 + pitch;
     const double* tY2 = tY1 + I.ylen;
     double T = vel_t(I.vel, I.Tper, 0);
-    C ux = (C)(tX1[x + GC] * tY1[y + GR] * T), uy = (C)(tX2[x + GC] * tY2[y + GR] * T);
+    C ux = (C)(12.0 * tX1[x + GC] * tY1[y + GR] * T), uy = (C)(12.0 * tX2[x + GC] * tY2[y + GR] * T);
     C ph = (C)c0, eta = (C)I.cd.eta;
     C uu = ux * ux + uy * uy;
     C v[9];

@@ -61,7 +61,9 @@ struct PairShape {
     static constexpr int TAB_N = 2 * W6 + 2 * H6;
     static constexpr unsigned TAB_BYTES = (TAB_N * sizeof(C) + 15) / 16 * 16;
     static constexpr int TAB_STRIDE = TAB_BYTES / sizeof(C);
-    static constexpr size_t BYTES = OFF_TAB + a128(TAB_BYTES) + 128;  // + alignment slack
+    // the Y tables times the two steps' time factors (time-dependent flows): Y1, Y2 for step t, then for t + 1
+    static constexpr size_t OFF_YT = OFF_TAB + a128(TAB_BYTES);
+    static constexpr size_t BYTES = OFF_YT + a128(4 * H6 * sizeof(C)) + 128;  // + alignment slack
 };
 
 // i reduced into [0, n); i lies within a few periods of the domain
@@ -73,21 +75,22 @@ __device__ __forceinline__ int wrap_near(int i, int n)
 }
 
 // mu (Eq. mu) and D = div(phi u) on a region of width W, height H, from phi on the region one node wider
-// (row stride PW); the velocity tables are indexed by the phi region's columns/rows shifted by `to`.
+// (row stride PW); the velocity tables (Y with the step's time factor) are indexed by the phi region's
+// columns/rows shifted by `to`.
 template <typename C, typename P, int W, int H, int PW, int NT>
 __device__ __forceinline__ void pair_mu_div(const P* ph, const C* sX1, const C* sX2, const C* sY1, const C* sY2,
-                                            int to, const Consts<C>& K0, bool model2, C T, C* s_mu, C* s_D)
+                                            int to, const Consts<C>& K0, bool model2, C* s_mu, C* s_D)
 {
     for_region<W, H, sizeof(C) == 4 ? PW : W, NT>([&](int e, int r, int c) {
         const P* q = ph + (r + 1) * PW + c + 1;
         const C ce = cvt<C>(q[0]);
         const C pE = cvt<C>(q[1]), pW = cvt<C>(q[-1]), pN = cvt<C>(q[PW]), pS = cvt<C>(q[-PW]);
         const C pNE = cvt<C>(q[PW + 1]), pNW = cvt<C>(q[PW - 1]), pSE = cvt<C>(q[-PW + 1]), pSW = cvt<C>(q[-PW - 1]);
-        s_mu[e] = node_mu(ce, pE, pW, pN, pS, pNE, pNW, pSE, pSW, K0.beta, K0.kappa, K0.phiA, K0.phiB);
+        s_mu[e] = mu9(ce, pE, pW, pN, pS, pNE, pNW, pSE, pSW, K0);
         if (model2) {
             const int tc = c + to, tr = r + to;  // the table index of the node's column/row minus one
-            s_D[e] = node_div(pE, pW, pN, pS, pNE, pNW, pSE, pSW, sX1[tc], sX1[tc + 2], sX2[tc], sX2[tc + 1],
-                              sX2[tc + 2], sY1[tr], sY1[tr + 1], sY1[tr + 2], sY2[tr], sY2[tr + 2], T);
+            s_D[e] = div9(pE, pW, pN, pS, pNE, pNW, pSE, pSW, sX1[tc], sX1[tc + 2], sX2[tc], sX2[tc + 1],
+                          sX2[tc + 2], sY1[tr], sY1[tr + 1], sY1[tr + 2], sY2[tr], sY2[tr + 2]);
         }
     });
 }
@@ -95,11 +98,11 @@ __device__ __forceinline__ void pair_mu_div(const P* ph, const C* sX1, const C* 
 // Force, equilibrium, source and collision at tau = 1 (Eqs. liangFi, mark3, geq, LB) on a region of width
 // W, height H; mu and D come from the region one node wider (stride MW), phi from the region two nodes
 // wider (stride PW), the velocity at table index (row, col) + tu.  The nine post-collision populations
-// are stored as planes of W * H values.
+// are stored as planes of W * H values, the axis directions in a quarter (collide9).
 template <typename C, typename P, int W, int H, int MW, int PW, int NT, bool kShift>
 __device__ __forceinline__ void pair_collide(const P* ph_reg, const C* s_mu, const C* s_D, const C* sX1,
                                              const C* sX2, const C* sY1, const C* sY2, int tu, const Consts<C>& K0,
-                                             bool model2, C T, C* s_post)
+                                             bool model2, C* s_post)
 {
     for_region<W, H, sizeof(C) == 4 ? MW : W, NT>([&](int e, int r, int c) {
         const int m = (r + 1) * MW + (c + 1);
@@ -110,13 +113,12 @@ __device__ __forceinline__ void pair_collide(const P* ph_reg, const C* s_mu, con
             grad9(s_D[m + 1], s_D[m - 1], s_D[m + MW], s_D[m - MW], s_D[m + MW + 1], s_D[m + MW - 1], s_D[m - MW + 1],
                   s_D[m - MW - 1], gDx, gDy);
         const C ph = cvt<C>(ph_reg[(r + 2) * PW + c + 2]);
-        C Fx, Fy;
-        node_force(ph, gmx, gmy, gDx, gDy, model2, K0.a, K0.b, K0.K, Fx, Fy);
-        const C ux = node_u(sX1[c + tu], sY1[r + tu], T), uy = node_u(sX2[c + tu], sY2[r + tu], T);
-        C g[9], post[9];
-#pragma unroll
-        for (int q = 0; q < 9; q++) g[q] = C(0);  // not read at tau = 1
-        collide9<C, true, kShift>(ph, s_mu[m], Fx, Fy, ux, uy, g, K0, post);
+        const C ux = node_u(sX1[c + tu], sY1[r + tu]), uy = node_u(sX2[c + tu], sY2[r + tu]);
+        C Px, Py, Jx, Jy, post[9];
+        node_flow(ph, ux, uy, K0, Px, Py);
+        node_force(ph, gmx, gmy, gDx, gDy, Px, Py, model2, K0, Jx, Jy);
+        collide9<C, true>(s_mu[m], ux, uy, Px, Py, Jx, Jy, nullptr, K0, post);
+        if (!kShift) post[0] = rest_add(post[0], ph, K0);
 #pragma unroll
         for (int q = 0; q < 9; q++) s_post[q * (W * H) + e] = post[q];
     });
@@ -134,7 +136,7 @@ __device__ __forceinline__ C pair_pull(const C* s_post, int r, int c, C& v0)
     v0 = s_post[p];
 #pragma unroll
     for (int q = 1; q < 9; q++) v[q] = s_post[q * NP + p - cy(q) * PW - cx(q)];
-    return stream_sum(v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8]);
+    return stream_sum_q(v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8]);
 }
 
 // phi(t+1) = phi(t) + g_0 + sum_q g_q on the float path: hi + lo absorbs the increment exactly (TwoSum),
@@ -164,6 +166,7 @@ struct PairSmem {
     C *mu, *D;   // mu and D of the step in progress
     C* post;     // post-collision populations of the step in progress, nine planes
     C *X1, *X2, *Y1, *Y2;  // velocity tables over the columns / rows of tile + 6
+    C* YT;       // Y1, Y2 times the time factor of step t, then of step t + 1
     __device__ explicit PairSmem(unsigned char* raw)
     {
         using L = PairShape<C, P, TX, TY>;
@@ -179,6 +182,7 @@ struct PairSmem {
         X2 = X1 + L::W6;
         Y1 = X2 + L::W6;
         Y2 = Y1 + L::H6;
+        YT = reinterpret_cast<C*>(base + L::OFF_YT);
     }
 };
 
@@ -238,10 +242,11 @@ struct PairLoad {
 
 // Steps t and t+1 of one tile from phi(t) and the tables in shared memory (loaded and synchronised by the
 // caller): phi(t+2) of the tile's domain nodes and their ghost images into phi_out (rb: the instance's first
-// domain node).  T0, T1: the flow's time factor at the two steps.  Ends without a barrier.
+// domain node).  timed: the flow depends on time; T0, T1: its time factor at the two steps (else 1).  Ends
+// without a barrier.
 template <typename C, typename P, int TX, int TY, int NT>
-__device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, const InstDev& I, C T0, C T1, int x0,
-                                           int y0, int pitch, long long rb, P* phi_out, float* lo_out)
+__device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, const InstDev& I, bool timed, C T0, C T1,
+                                           int x0, int y0, int pitch, long long rb, P* phi_out, float* lo_out)
 {
     using L = PairShape<C, P, TX, TY>;
     constexpr bool kFF = L::FF;
@@ -251,11 +256,24 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
     const Consts<C>& K0 = consts<C>(I);
     const bool model2 = I.model == 2;
 
+    const C *Ya1 = S.Y1, *Ya2 = S.Y2, *Yb1 = S.Y1, *Yb2 = S.Y2;  // the Y tables of the two steps
+    if (timed) {
+        for (int e = threadIdx.x; e < 2 * L::H6; e += NT) {
+            const C y = S.Y1[e];
+            S.YT[e] = op_mul(y, T0);
+            S.YT[2 * L::H6 + e] = op_mul(y, T1);
+        }
+        __syncthreads();
+        Ya1 = S.YT;
+        Ya2 = Ya1 + L::H6;
+        Yb1 = Ya2 + L::H6;
+        Yb2 = Yb1 + L::H6;
+    }
+
     // step t: mu, D on tile + 5; collision on tile + 4; streaming to phi(t+1) on tile + 3
-    pair_mu_div<C, P, L::W5, L::H5, W6, NT>(S.phi0, S.X1, S.X2, S.Y1, S.Y2, 0, K0, model2, T0, S.mu, S.D);
+    pair_mu_div<C, P, L::W5, L::H5, W6, NT>(S.phi0, S.X1, S.X2, Ya1, Ya2, 0, K0, model2, S.mu, S.D);
     __syncthreads();
-    pair_collide<C, P, L::W4, L::H4, L::W5, W6, NT, kShift>(S.phi0, S.mu, S.D, S.X1, S.X2, S.Y1, S.Y2, 2, K0, model2, T0,
-                                                           S.post);
+    pair_collide<C, P, L::W4, L::H4, L::W5, W6, NT, kShift>(S.phi0, S.mu, S.D, S.X1, S.X2, Ya1, Ya2, 2, K0, model2, S.post);
     __syncthreads();
     for_region<W3, L::H3, sizeof(C) == 4 ? L::W4 : W3, NT>([&](int e, int r, int c) {
         C v0;
@@ -267,10 +285,9 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
     __syncthreads();
 
     // step t+1: mu, D on tile + 2; collision on tile + 1; streaming to phi(t+2) on the tile
-    pair_mu_div<C, P, L::W2, L::H2, W3, NT>(S.hi1, S.X1, S.X2, S.Y1, S.Y2, 3, K0, model2, T1, S.mu, S.D);
+    pair_mu_div<C, P, L::W2, L::H2, W3, NT>(S.hi1, S.X1, S.X2, Yb1, Yb2, 3, K0, model2, S.mu, S.D);
     __syncthreads();
-    pair_collide<C, P, L::W1, L::H1, L::W2, W3, NT, kShift>(S.hi1, S.mu, S.D, S.X1, S.X2, S.Y1, S.Y2, 5, K0, model2, T1,
-                                                           S.post);
+    pair_collide<C, P, L::W1, L::H1, L::W2, W3, NT, kShift>(S.hi1, S.mu, S.D, S.X1, S.X2, Yb1, Yb2, 5, K0, model2, S.post);
     __syncthreads();
     const int nx = I.nx, ny = I.ny;
     for_region<TX, TY, sizeof(C) == 4 ? L::W1 : TX, NT>([&](int e, int r, int c) {
@@ -381,7 +398,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __
                 __syncthreads();
                 if (s_abort) break;
             }
-            pair_steps<C, P, TX, TY, NT>(S, I, s_T[0], s_T[1], x0, y0, a.pitch, rb, a.phi_out, a.lo_out);
+            pair_steps<C, P, TX, TY, NT>(S, I, a.need_time, s_T[0], s_T[1], x0, y0, a.pitch, rb, a.phi_out, a.lo_out);
         }
     } else {
         // thread 0: tile t's instance (copied when it changes) and origin
@@ -434,7 +451,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __
                 __syncthreads();
                 if (s_abort) break;
             }
-            pair_steps<C, P, TX, TY, NT>(S, s_I, s_T[0], s_T[1], s_x0, s_y0, a.pitch, rb, a.phi_out, a.lo_out);
+            pair_steps<C, P, TX, TY, NT>(S, s_I, a.need_time, s_T[0], s_T[1], s_x0, s_y0, a.pitch, rb, a.phi_out, a.lo_out);
         }
     }
 

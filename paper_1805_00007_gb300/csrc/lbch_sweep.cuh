@@ -8,7 +8,9 @@
 //
 //   * a warp owns 64 consecutive columns, two per lane (a = 2 lane, b = 2 lane + 1, from domain column
 //     x0 - 4); its 56 middle columns (lanes 2..29) are output, the four on each side are halo;
-//   * the left neighbour of a and the right neighbour of b come from the adjacent lanes by shuffles;
+//   * the stencils are taken column first (lbch_kernels.cuh): each lane forms the column values of its two
+//     columns from the rows in its registers, and what the combination along the row needs of the left
+//     neighbour of a and the right neighbour of b comes from the adjacent lanes by shuffles;
 //   * the rows below stay in registers: iteration j loads phi of row yf = wy0 - 3 + j, computes mu and D
 //     of row yf - 1, collides row yf - 2 and completes phi(t+1) of row yf - 3;
 //   * streaming needs only three values from each side: the populations 1, 5, 8 that arrive from the
@@ -114,12 +116,12 @@ template <typename C> __device__ __forceinline__ C from_right(C v) { return __sh
 // One row of the sweep.  A slot is reused every third row, so each field lives at most three rows.
 template <typename C>
 struct SwRow {
-    C pL, pa, pb, pR;              // phi: left neighbour of a, a, b, right neighbour of b
-    C mL, ma, mb, mR;              // mu, the same four columns
-    C dL, da, db, dR;              // D = div(phi u)
+    C pa, pb;                      // phi
+    C ma, mb;                      // mu
+    C da, db;                      // D = div(phi u)
     C y1, y2;                      // the Y velocity tables of the row
-    C u5a, u5b, u2a, u2b, u6a, u6b;         // g*_5, g*_2, g*_6 of the row: they stream to the row above
-    C Ra, Rb, Ca, Cb, La, Lb, v0a, v0b;     // partial sums of the populations arriving at the row
+    C u5a, u5b, u2a, u2b, u6a, u6b;         // g*_5, a quarter of g*_2, g*_6 of the row: they stream to the row above
+    C Ra, Rb, Ca, Cb, La, Lb, v0a, v0b;     // partial sums of the populations arriving at the row (C in a quarter)
     C e4a, e4b, e7a, e7b, e8a, e8b;         // at a top wall row: g_4, g_7, g_8 by bounce-back
     C n0a, n0b, n1a, n1b, n2a, n2b, n3a, n3b, n4a, n4b, n5a, n5b, n6a, n6b, n7a, n7b, n8a, n8b;  // GEN: g(t+1) of the row
 };
@@ -219,7 +221,7 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
     // instance's stored band, one row of the warp per lane.
     int k_t = 0, x0 = 0, y0 = 0;
     bool w_t = false;  // the tile needs the wall body
-    C X1m, X1a, X1b, X1p, X2m, X2a, X2b, X2p, ly1, ly2;
+    C X1a, X1b, X2a, X2b, ly1, ly2;
     auto locate = [&](int t) {
         int tab_t, ylen;
         if constexpr (SINGLE) {
@@ -242,9 +244,9 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
         const C* tX2 = tX1 + a.pitch;
         const C* tY1 = tX2 + a.pitch;
         const int sa = x0 + 2 * lane;
-        const int cm = max(sa - 1, 0), ca = min(sa, a.pitch - 1), cb = min(sa + 1, a.pitch - 1), cp = min(sa + 2, a.pitch - 1);
-        X1m = tX1[cm]; X1a = tX1[ca]; X1b = tX1[cb]; X1p = tX1[cp];
-        X2m = tX2[cm]; X2a = tX2[ca]; X2b = tX2[cb]; X2p = tX2[cp];
+        const int ca = min(sa, a.pitch - 1), cb = min(sa + 1, a.pitch - 1);
+        X1a = tX1[ca]; X1b = tX1[cb];
+        X2a = tX2[ca]; X2b = tX2[cb];
         const int yk = min(max(y0 + warp * TY - 3 + lane + GR, 0), ylen - 1);
         ly1 = tY1[yk];
         ly2 = tY1[ylen + yk];
@@ -317,12 +319,11 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
         const int wy0 = y0 + warp * TY;  // the warp's first output row
         if (wy0 >= ny) return;
         const Consts<C>& K0 = consts<C>(I);
-        const C beta = K0.beta, kappa = K0.kappa, phiA = K0.phiA, phiB = K0.phiB;
-        const C ra = K0.a, rb = K0.b, K = K0.K;
         const bool model2 = M3 ? I.model >= 2 : I.model == 2;  // D = div(phi u) is needed (Models II, III)
         [[maybe_unused]] const bool model3 = M3 && I.model == 3;
         [[maybe_unused]] const bool first = M3 && s_time + a.t_off == 0;  // no H(t - 1) at the first step
         const C T = s_T;
+        const C my1 = op_mul(ly1, T), my2 = op_mul(ly2, T);  // the warp's rows' Y tables with the time factor
         const int pitch = a.pitch;
         // this lane's column pair in the box, from the warp's first row (box row warp TY = domain wy0 - 3)
         const P* box = reinterpret_cast<const P*>(stage(s)) + warp * TY * BW + 2 * lane;
@@ -375,23 +376,22 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
                 const P2 v = *reinterpret_cast<const P2*>(box + j * BW);
                 A.pa = cvt<C>(v.x);
                 A.pb = cvt<C>(v.y);
-                A.pL = from_left(A.pb);
-                A.pR = from_right(A.pa);
-                A.y1 = __shfl_sync(0xffffffffu, ly1, j);
-                A.y2 = __shfl_sync(0xffffffffu, ly2, j);
+                A.y1 = __shfl_sync(0xffffffffu, my1, j);
+                A.y2 = __shfl_sync(0xffffffffu, my2, j);
             }
             if (MU) {
-                B.ma = node_mu(B.pa, B.pb, B.pL, A.pa, Cs.pa, A.pb, A.pL, Cs.pb, Cs.pL, beta, kappa, phiA, phiB);
-                B.mb = node_mu(B.pb, B.pR, B.pa, A.pb, Cs.pb, A.pR, A.pa, Cs.pR, Cs.pa, beta, kappa, phiA, phiB);
-                B.mL = from_left(B.mb);
-                B.mR = from_right(B.ma);
+                C dla, dlb;
+                const C za = node_z(Cs.pa, B.pa, A.pa, dla), zb = node_z(Cs.pb, B.pb, A.pb, dlb);
+                const C zL = from_left(zb), zR = from_right(za);
+                B.ma = node_mu(B.pa, dla, za, zb, zL, K0);
+                B.mb = node_mu(B.pb, dlb, zb, zR, za, K0);
                 if (model2) {
-                    B.da = node_div(B.pb, B.pL, A.pa, Cs.pa, A.pb, A.pL, Cs.pb, Cs.pL, X1m, X1b, X2m, X2a, X2b,
-                                    Cs.y1, B.y1, A.y1, Cs.y2, A.y2, T);
-                    B.db = node_div(B.pR, B.pa, A.pb, Cs.pb, A.pR, A.pa, Cs.pR, Cs.pa, X1a, X1p, X2a, X2b, X2p,
-                                    Cs.y1, B.y1, A.y1, Cs.y2, A.y2, T);
-                    B.dL = from_left(B.db);
-                    B.dR = from_right(B.da);
+                    const C y14 = op_mul(C(4), B.y1);
+                    C Ea, Wa, Eb, Wb;
+                    const C fa = node_flux(Cs.pa, B.pa, A.pa, X1a, X2a, Cs.y1, y14, A.y1, Cs.y2, A.y2, Ea, Wa);
+                    const C fb = node_flux(Cs.pb, B.pb, A.pb, X1b, X2b, Cs.y1, y14, A.y1, Cs.y2, A.y2, Eb, Wb);
+                    B.da = node_div(fa, Eb, from_left(Wb));
+                    B.db = node_div(fb, from_right(Ea), Wa);
                 }
             }
             const int yc = yf - 2;
@@ -425,19 +425,25 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
                     if constexpr (WALLS) {
                         // next to a wall, mu and D of the ghost row take the values of the mirror row (yc);
                         // the ghost row's own values are used by no other node
-                        if (yc == 0) { A.mL = Cs.mL; A.ma = Cs.ma; A.mb = Cs.mb; A.mR = Cs.mR;
-                                       A.dL = Cs.dL; A.da = Cs.da; A.db = Cs.db; A.dR = Cs.dR; }
-                        if (yc == ny - 1) { B.mL = Cs.mL; B.ma = Cs.ma; B.mb = Cs.mb; B.mR = Cs.mR;
-                                            B.dL = Cs.dL; B.da = Cs.da; B.db = Cs.db; B.dR = Cs.dR; }
+                        if (yc == 0) { A.ma = Cs.ma; A.mb = Cs.mb; A.da = Cs.da; A.db = Cs.db; }
+                        if (yc == ny - 1) { B.ma = Cs.ma; B.mb = Cs.mb; B.da = Cs.da; B.db = Cs.db; }
                     }
+                    // 12 grad: of the pair (a, b), from the column values w and d of both and of their neighbours
+                    auto grad_pair = [&](C sa_, C ca_, C na_, C sb_, C cb_, C nb_, C& gxa, C& gya, C& gxb, C& gyb) {
+                        const C wa = node_w(sa_, ca_, na_), wb = node_w(sb_, cb_, nb_), da = na_ - sa_, db = nb_ - sb_;
+                        gxa = wb - from_left(wb);
+                        gxb = from_right(wa) - wa;
+                        gya = node_gy(from_left(db), da, db);
+                        gyb = node_gy(da, db, from_right(da));
+                    };
                     C gmxa, gmya, gmxb, gmyb, gDxa = C(0), gDya = C(0), gDxb = C(0), gDyb = C(0);
-                    grad9(Cs.mb, Cs.mL, B.ma, A.ma, B.mb, B.mL, A.mb, A.mL, gmxa, gmya);
-                    grad9(Cs.mR, Cs.ma, B.mb, A.mb, B.mR, B.ma, A.mR, A.ma, gmxb, gmyb);
-                    if (model2) {
-                        grad9(Cs.db, Cs.dL, B.da, A.da, B.db, B.dL, A.db, A.dL, gDxa, gDya);
-                        grad9(Cs.dR, Cs.da, B.db, A.db, B.dR, B.da, A.dR, A.da, gDxb, gDyb);
-                    }
-                    C Fxa, Fya, Fxb, Fyb;
+                    grad_pair(A.ma, Cs.ma, B.ma, A.mb, Cs.mb, B.mb, gmxa, gmya, gmxb, gmyb);
+                    if (model2) grad_pair(A.da, Cs.da, B.da, A.db, Cs.db, B.db, gDxa, gDya, gDxb, gDyb);
+                    const C uxa = node_u(X1a, Cs.y1), uya = node_u(X2a, Cs.y2);
+                    const C uxb = node_u(X1b, Cs.y1), uyb = node_u(X2b, Cs.y2);
+                    C Pxa, Pya, Pxb, Pyb, Jxa, Jya, Jxb, Jyb;
+                    node_flow(Cs.pa, uxa, uya, K0, Pxa, Pya);
+                    node_flow(Cs.pb, uxb, uyb, K0, Pxb, Pyb);
                     if (M3 && model3) {
                         // H(t - 1) at the collided nodes: rows -1 .. ny hold it (images one deep); other rows
                         // and columns past the stored ones collide for no output and read nothing
@@ -448,23 +454,23 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
                         const C Hpxb = hrow && sa + 1 < pitch ? a.H_in[hn + 1] : C(0);
                         const C Hpyb = hrow && sa + 1 < pitch ? a.H_in[a.H_plane + hn + 1] : C(0);
                         C Hxa, Hya, Hxb, Hyb;
-                        node_force_full(Cs.pa, gmxa, gmya, gDxa, gDya, Hpxa, Hpya, first, ra, rb, K, K0.cF1, K0.cmu,
-                                        Fxa, Fya, Hxa, Hya);
-                        node_force_full(Cs.pb, gmxb, gmyb, gDxb, gDyb, Hpxb, Hpyb, first, ra, rb, K, K0.cF1, K0.cmu,
-                                        Fxb, Fyb, Hxb, Hyb);
+                        node_force_full(Cs.pa, gmxa, gmya, gDxa, gDya, Hpxa, Hpya, first, Pxa, Pya, K0, Jxa, Jya, Hxa, Hya);
+                        node_force_full(Cs.pb, gmxb, gmyb, gDxb, gDyb, Hpxb, Hpyb, first, Pxb, Pyb, K0, Jxb, Jyb, Hxb, Hyb);
                         if (yc >= wy0 && yc < wy0 + TY && yc < ny) {  // the warp's own nodes
                             if (va) store_h(a.H_out, a.H_plane, (int)row0, pitch, nx, ny, I.walls, xa, yc, Hxa, Hya);
                             if (vb) store_h(a.H_out, a.H_plane, (int)row0, pitch, nx, ny, I.walls, xb, yc, Hxb, Hyb);
                         }
                     } else {
-                        node_force(Cs.pa, gmxa, gmya, gDxa, gDya, model2, ra, rb, K, Fxa, Fya);
-                        node_force(Cs.pb, gmxb, gmyb, gDxb, gDyb, model2, ra, rb, K, Fxb, Fyb);
+                        node_force(Cs.pa, gmxa, gmya, gDxa, gDya, Pxa, Pya, model2, K0, Jxa, Jya);
+                        node_force(Cs.pb, gmxb, gmyb, gDxb, gDyb, Pxb, Pyb, model2, K0, Jxb, Jyb);
                     }
-                    C pa_[9], pb_[9];
-                    collide9<C, !GEN, kShift, !GEN>(Cs.pa, Cs.ma, Fxa, Fya, node_u(X1a, Cs.y1, T), node_u(X2a, Cs.y2, T), ga,
-                                              K0, pa_);
-                    collide9<C, !GEN, kShift, !GEN>(Cs.pb, Cs.mb, Fxb, Fyb, node_u(X1b, Cs.y1, T), node_u(X2b, Cs.y2, T), gb,
-                                              K0, pb_);
+                    C pa_[9], pb_[9];  // without the populations: 1..4 in a quarter
+                    collide9<C, !GEN>(Cs.ma, uxa, uya, Pxa, Pya, Jxa, Jya, ga, K0, pa_);
+                    collide9<C, !GEN>(Cs.mb, uxb, uyb, Pxb, Pyb, Jxb, Jyb, gb, K0, pb_);
+                    if constexpr (!kShift) {
+                        pa_[0] = rest_add(pa_[0], Cs.pa, K0);
+                        pb_[0] = rest_add(pb_[0], Cs.pb, K0);
+                    }
                     if constexpr (GEN && kHalf) {
                         // the streamed populations are stored in half: they travel rounded.  g*_0 stays at the
                         // node, in float, and takes what the rounded ones leave of phi (g*_0 - phi = -sum of
@@ -496,15 +502,15 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
                         A.n8a = from_left(pb_[8]); A.n8b = pa_[8];
                         if constexpr (WALLS) {
                             if (yc == 0) {  // bottom wall: 2, 5, 6 of this row bounce back at the node
-                                const C uxa = node_u(X1a, tW[0], T), uya = node_u(X2a, tW[2], T);
-                                const C uxb = node_u(X1b, tW[0], T), uyb = node_u(X2b, tW[2], T);
+                                const C uxa = wall_u(X1a, tW[0], T), uya = wall_u(X2a, tW[2], T);
+                                const C uxb = wall_u(X1b, tW[0], T), uyb = wall_u(X2b, tW[2], T);
                                 Cs.n2a = bounce<C, 2>(pa_[4], Cs.pa, uxa, uya); Cs.n2b = bounce<C, 2>(pb_[4], Cs.pb, uxb, uyb);
                                 Cs.n5a = bounce<C, 5>(pa_[7], Cs.pa, uxa, uya); Cs.n5b = bounce<C, 5>(pb_[7], Cs.pb, uxb, uyb);
                                 Cs.n6a = bounce<C, 6>(pa_[8], Cs.pa, uxa, uya); Cs.n6b = bounce<C, 6>(pb_[8], Cs.pb, uxb, uyb);
                             }
                             if (yc == ny - 1) {  // top wall: 4, 7, 8 of this row
-                                const C uxa = node_u(X1a, tW[1], T), uya = node_u(X2a, tW[3], T);
-                                const C uxb = node_u(X1b, tW[1], T), uyb = node_u(X2b, tW[3], T);
+                                const C uxa = wall_u(X1a, tW[1], T), uya = wall_u(X2a, tW[3], T);
+                                const C uxb = wall_u(X1b, tW[1], T), uyb = wall_u(X2b, tW[3], T);
                                 Cs.n4a = bounce<C, 4>(pa_[2], Cs.pa, uxa, uya); Cs.n4b = bounce<C, 4>(pb_[2], Cs.pb, uxb, uyb);
                                 Cs.n7a = bounce<C, 7>(pa_[5], Cs.pa, uxa, uya); Cs.n7b = bounce<C, 7>(pb_[5], Cs.pb, uxb, uyb);
                                 Cs.n8a = bounce<C, 8>(pa_[6], Cs.pa, uxa, uya); Cs.n8b = bounce<C, 8>(pb_[6], Cs.pb, uxb, uyb);
@@ -514,30 +520,31 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
                     Cs.u5a = pa_[5]; Cs.u5b = pb_[5];
                     Cs.u2a = pa_[2]; Cs.u2b = pb_[2];
                     Cs.u6a = pa_[6]; Cs.u6b = pb_[6];
-                    // (g_1 + g_5) and (g_3 + g_6) at their source nodes; g_2 from the row below
-                    Cs.Ra = pa_[1] + A.u5a; Cs.Rb = pb_[1] + A.u5b;
-                    Cs.La = pa_[3] + A.u6a; Cs.Lb = pb_[3] + A.u6b;
+                    // (g_1 + g_5) and (g_3 + g_6) at their source nodes; g_2 (a quarter of it) from the row below
+                    Cs.Ra = op_fma(C(4), pa_[1], A.u5a); Cs.Rb = op_fma(C(4), pb_[1], A.u5b);
+                    Cs.La = op_fma(C(4), pa_[3], A.u6a); Cs.Lb = op_fma(C(4), pb_[3], A.u6b);
                     Cs.Ca = A.u2a; Cs.Cb = A.u2b;
                     Cs.v0a = pa_[0];
                     Cs.v0b = pb_[0];
                     if constexpr (WALLS) {
                         if (yc == 0) {
                             // bottom wall row: 2, 5, 6 would come from the ghost row; they bounce back at the
-                            // node, so the sums from the sides are formed here, at the destination
-                            const C uxa = node_u(X1a, tW[0], T), uya = node_u(X2a, tW[2], T);
-                            const C uxb = node_u(X1b, tW[0], T), uyb = node_u(X2b, tW[2], T);
-                            Cs.Ra = from_left(pb_[1]) + bounce<C, 5>(pa_[7], Cs.pa, uxa, uya);
-                            Cs.Rb = pa_[1] + bounce<C, 5>(pb_[7], Cs.pb, uxb, uyb);
-                            Cs.La = pb_[3] + bounce<C, 6>(pa_[8], Cs.pa, uxa, uya);
-                            Cs.Lb = from_right(pa_[3]) + bounce<C, 6>(pb_[8], Cs.pb, uxb, uyb);
-                            Cs.Ca = bounce<C, 2>(pa_[4], Cs.pa, uxa, uya);
-                            Cs.Cb = bounce<C, 2>(pb_[4], Cs.pb, uxb, uyb);
+                            // node, so the sums from the sides are formed here, at the destination (C in full)
+                            const C uxa = wall_u(X1a, tW[0], T), uya = wall_u(X2a, tW[2], T);
+                            const C uxb = wall_u(X1b, tW[0], T), uyb = wall_u(X2b, tW[2], T);
+                            Cs.Ra = op_fma(C(4), from_left(pb_[1]), bounce<C, 5>(pa_[7], Cs.pa, uxa, uya));
+                            Cs.Rb = op_fma(C(4), pa_[1], bounce<C, 5>(pb_[7], Cs.pb, uxb, uyb));
+                            Cs.La = op_fma(C(4), pb_[3], bounce<C, 6>(pa_[8], Cs.pa, uxa, uya));
+                            Cs.Lb = op_fma(C(4), from_right(pa_[3]), bounce<C, 6>(pb_[8], Cs.pb, uxb, uyb));
+                            Cs.Ca = bounce<C, 2>(op_mul(C(4), pa_[4]), Cs.pa, uxa, uya);
+                            Cs.Cb = bounce<C, 2>(op_mul(C(4), pb_[4]), Cs.pb, uxb, uyb);
                         }
                         if (yc == ny - 1) {
-                            // top wall row: 4, 7, 8 would come from the ghost row above
-                            const C uxa = node_u(X1a, tW[1], T), uya = node_u(X2a, tW[3], T);
-                            const C uxb = node_u(X1b, tW[1], T), uyb = node_u(X2b, tW[3], T);
-                            Cs.e4a = bounce<C, 4>(pa_[2], Cs.pa, uxa, uya); Cs.e4b = bounce<C, 4>(pb_[2], Cs.pb, uxb, uyb);
+                            // top wall row: 4, 7, 8 would come from the ghost row above (e4 in full)
+                            const C uxa = wall_u(X1a, tW[1], T), uya = wall_u(X2a, tW[3], T);
+                            const C uxb = wall_u(X1b, tW[1], T), uyb = wall_u(X2b, tW[3], T);
+                            Cs.e4a = bounce<C, 4>(op_mul(C(4), pa_[2]), Cs.pa, uxa, uya);
+                            Cs.e4b = bounce<C, 4>(op_mul(C(4), pb_[2]), Cs.pb, uxb, uyb);
                             Cs.e7a = bounce<C, 7>(pa_[5], Cs.pa, uxa, uya); Cs.e7b = bounce<C, 7>(pb_[5], Cs.pb, uxb, uyb);
                             Cs.e8a = bounce<C, 8>(pa_[6], Cs.pa, uxa, uya); Cs.e8b = bounce<C, 8>(pb_[6], Cs.pb, uxb, uyb);
                         }
@@ -624,25 +631,25 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
             if (!GEN && OUT) {
                 // phi(t+1) of row yo = yf - 3 (slot A), with g*_4, g*_7, g*_8 of row yo + 1 just computed
                 const int yo = yf - 3;
-                C Ra, Rb, Ca, Cb, La, Lb;
+                // R, L: the sums from the left and the right; RC = R + C with C = g_2 + g_4
+                C RCa, RCb, La, Lb;
                 if (WALLS && yo == ny - 1) {
                     // top wall row (no collision above): the sums (g_1 + g_5), (g_3 + g_6) cross to their
                     // destinations, where the bounced-back 8, 7 and 4 complete them
-                    Ra = from_left(A.Rb) + A.e8a; Rb = A.Ra + A.e8b;
+                    RCa = (from_left(A.Rb) + A.e8a) + op_fma(C(4), A.Ca, A.e4a);
+                    RCb = (A.Ra + A.e8b) + op_fma(C(4), A.Cb, A.e4b);
                     La = A.Lb + A.e7a; Lb = from_right(A.La) + A.e7b;
-                    Ca = A.Ca + A.e4a; Cb = A.Cb + A.e4b;
                 } else if (WALLS && yo == 0) {
                     // bottom wall row: the sums are already at the destinations
-                    Ra = A.Ra + from_left(p8b); Rb = A.Rb + p8a;
+                    RCa = (A.Ra + from_left(p8b)) + op_fma(C(4), p4a, A.Ca);
+                    RCb = (A.Rb + p8a) + op_fma(C(4), p4b, A.Cb);
                     La = A.La + p7b; Lb = A.Lb + from_right(p7a);
-                    Ca = A.Ca + p4a; Cb = A.Cb + p4b;
                 } else {
                     const C Rsa = A.Ra + p8a, Rsb = A.Rb + p8b, Lsa = A.La + p7a, Lsb = A.Lb + p7b;
-                    Ra = from_left(Rsb); Rb = Rsa;
+                    RCa = op_fma(C(4), A.Ca + p4a, from_left(Rsb)); RCb = op_fma(C(4), A.Cb + p4b, Rsa);
                     La = Lsb; Lb = from_right(Lsa);
-                    Ca = A.Ca + p4a; Cb = A.Cb + p4b;
                 }
-                const C suma = (Ra + Ca) + La, sumb = (Rb + Cb) + Lb;  // the grouping of stream_sum
+                const C suma = RCa + La, sumb = RCb + Lb;  // the grouping of stream_sum
                 P hia, hib;
                 float loa = 0.0f, lob = 0.0f;
                 if constexpr (FF) {
