@@ -188,6 +188,8 @@ cudaError_t launch_step_v(lbch_handle* h, int parity)
     a.t_off = h->t_off;
     a.t_adv = h->t_adv;
     a.need_time = h->need_time;
+    a.Tf = launch_T(h);
+    a.read_n = launch_reads_n(h);
     // a programmatic dependent of the previous launch in the stream (the kernel waits on it before it
     // touches memory that launch writes), so its launch and prologue overlap the previous step's tail
     cudaLaunchConfig_t cfg = {};
@@ -402,6 +404,16 @@ cudaError_t launch_step(lbch_handle* h, int parity)
              : k == 1 ? launch_step_t<float, __half, float, 32, 8>(h, parity)
              : k == 2 ? launch_step_t<float, __half, float, 16, 8>(h, parity) : launch_step_t<float, __half, float, 32, 16, 768>(h, parity);
     }
+}
+
+// The table of time factors for the next `steps` (at most kTimeSteps) steps; the launches that follow name their row
+// of it in h->t_row.  An ordinary stream-ordered launch: the steps that read the previous table are complete.
+cudaError_t time_table(lbch_handle* h, int steps)
+{
+    if (!h->timed) return cudaSuccess;
+    const int n = steps * h->n_inst;
+    time_table_kernel<<<(n + 127) / 128, 128, 0, h->stream>>>(h->d_inst, h->n_inst, h->ctl, steps, h->d_T);
+    return cudaGetLastError();
 }
 
 // Two steps by one launch of the two-step kernel, outside a graph (the launch advances the counter by
@@ -678,6 +690,7 @@ void release(lbch_handle* h)
     }
     dfree(h, h->d_node_begin);
     dfree(h, h->d_tabs);
+    dfree(h, h->d_T);
     dfree(h, h->phi0);
     dfree(h, h->ctl);
     dfree(h, h->partials);
@@ -1060,9 +1073,10 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     h->n_inst = n_inst;
     for (int k = 0; k < n_inst; k++) h->model3 = h->model3 || params[k].model == 3;
     for (int k = 0; k < n_inst; k++) h->walls = h->walls || params[k].walls != 0;
-    for (int k = 0; k < n_inst; k++)  // the flows with a time factor (vel_t), and Model III's first step
-        h->need_time = h->need_time || params[k].model == 3 || params[k].vel == LBCH_VEL_VORTEX ||
-                       params[k].vel == LBCH_VEL_DEFORM || params[k].vel == LBCH_VEL_REV_SHEAR;
+    for (int k = 0; k < n_inst; k++)  // the flows with a time factor (vel_t)
+        h->timed = h->timed || params[k].vel == LBCH_VEL_VORTEX || params[k].vel == LBCH_VEL_DEFORM ||
+                   params[k].vel == LBCH_VEL_REV_SHEAR;
+    h->need_time = h->timed || h->model3;  // Model III: its first step
     h->g_elem = prec == LBCH_F64 ? 8 : (prec == LBCH_F32 ? 4 : 2);
     h->phi_elem = prec == LBCH_F64 ? 8 : 4;  // the float path adds a float low part
     h->nq = prec == LBCH_F16S ? 8 : 9;
@@ -1238,6 +1252,7 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     CKI(dalloc(h, &h->d_tabs, sizeof(double) * tabs.size()));
     CKI(dalloc(h, &h->d_tabs_f, sizeof(float) * tabs_f.size()));
     CKI(dalloc(h, &h->ctl, sizeof(Ctl)));
+    if (h->timed) CKI(dalloc(h, &h->d_T, sizeof(double) * kTimeSteps * (size_t)n_inst));
     long long max_nodes = 0;
     for (auto& d : h->inst) max_nodes = std::max(max_nodes, (long long)d.nx * d.ny);
     h->chunks = (int)std::min<long long>(1024, (max_nodes + RED_NT * 8 - 1) / (RED_NT * 8));
@@ -1378,6 +1393,8 @@ lbch_status lb_ch_step(lbch_handle* h, long nsteps)
         return fail(LBCH_EINVAL, "a slab handle advances one step per call: import its halos before every step");
     static const bool no_graph = std::getenv("LBCH_NO_GRAPH") != nullptr;
     const bool two = use_pair(h);
+    static_assert(kTimeSteps >= kGraphBig, "a graph's time factors fit one table");
+    int rows = 0, row = 0;  // single launches: the rows of the current table of time factors, and the next one's
     while (nsteps > 0) {
         int parity = cur_buf(h);
         if (!no_graph && !h->debug_skip && nsteps >= kGraphChunk) {
@@ -1391,12 +1408,15 @@ lbch_status lb_ch_step(lbch_handle* h, long nsteps)
                 // the two-step kernel, launch s takes steps 2s and 2s + 1; the chunk's launch count is even,
                 // so the graph ends in the buffer it starts from, as the one-step graph does.
                 const int per = two ? 2 : 1, launches = chunk / per;
+                e = time_table(h, chunk);
                 for (int s = 0; s < launches && e == cudaSuccess; s++) {
                     h->t_off = s * per;
+                    h->t_row = s * per;
                     h->t_adv = s == launches - 1 ? chunk : 0;
                     e = two ? lbch_launch_pair(h, parity ^ (s & 1)) : launch_step(h, parity ^ (s & 1));
                 }
                 h->t_off = 0;
+                h->t_row = -1;
                 h->t_adv = 1;
                 cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
                 if (e != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(e, "step launch during capture"); }
@@ -1408,13 +1428,27 @@ lbch_status lb_ch_step(lbch_handle* h, long nsteps)
             CK(cudaGraphLaunch(gx, h->stream));
             h->n += chunk;
             nsteps -= chunk;
-        } else if (two && nsteps >= 2) {
-            CK(launch_pair_now(h));
-            nsteps -= 2;
         } else {
-            CK(launch_step(h, parity));
-            h->n += 1;
-            nsteps -= 1;
+            // a few last steps form their time factors themselves: the table's own launch costs about as much as
+            // the factors of three launches
+            const int per = two && nsteps >= 2 ? 2 : 1;
+            if (row + per > rows && h->timed && nsteps > 3 * per) {
+                rows = (int)std::min<long>(nsteps, kTimeSteps);
+                row = 0;
+                CK(time_table(h, rows));
+            }
+            h->t_row = row + per <= rows ? row : -1;
+            row += per;
+            cudaError_t e = cudaSuccess;
+            if (per == 2) {
+                e = launch_pair_now(h);
+            } else {
+                e = launch_step(h, parity);
+                if (e == cudaSuccess) h->n += 1;
+            }
+            h->t_row = -1;
+            CK(e);
+            nsteps -= per;
         }
     }
     return LBCH_OK;
@@ -1693,13 +1727,17 @@ lbch_status lb_ch_step_taped(lbch_handle* h, long nsteps, void* tape)
             cudaGraph_t g = nullptr;
             CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
             cudaError_t e = cudaSuccess;
+            const bool table = nsteps <= kTimeSteps;
+            if (table) e = time_table(h, (int)nsteps);
             for (long k = 0; k < nsteps && e == cudaSuccess; k++) {
                 e = tape_launch(h, parity ^ (int)(k & 1), t + (size_t)k * stride);
                 h->t_off = (int)k;
+                h->t_row = table ? (int)k : -1;
                 h->t_adv = k == nsteps - 1 ? (int)nsteps : 0;
                 if (e == cudaSuccess) e = launch_step(h, parity ^ (int)(k & 1));
             }
             h->t_off = 0;
+            h->t_row = -1;
             h->t_adv = 1;
             cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
             if (e != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(e, "taped step launch during capture"); }

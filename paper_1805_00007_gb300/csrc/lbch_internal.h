@@ -80,6 +80,9 @@ struct lbch_handle {
     long long n = 0;            // host mirror of the step index
     int flip = 0;               // the state of step n is in buffer (n & 1) ^ flip (two-step launches toggle it)
     int t_off = 0, t_adv = 1;   // the next launch's step offset and counter advance (see Ctl)
+    bool timed = false;         // an instance's flow has a time factor
+    double* d_T = nullptr;      // timed handles: the time factors of a batch of up to kTimeSteps steps
+    int t_row = -1;             // the next launch's row of d_T, or -1: the launch forms its time factors itself
     int debug_skip = 0;
     cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [chunk size][starting parity]
     struct TapeGraph {          // a captured taped replay (lb_ch_step_taped) for one starting parity
@@ -108,6 +111,14 @@ template <> inline const float* tables<float>(lbch_handle* h) { return h->d_tabs
 
 // The buffer (0 or 1 of each ping-pong pair) holding the state of the current step.
 inline int cur_buf(const lbch_handle* h) { return (int)(h->n & 1) ^ h->flip; }
+
+constexpr int kTimeSteps = 512;  // steps per table of time factors (a big graph's; longer batches form several)
+// The time factors of the next launch, and whether it reads the step index.
+inline const double* launch_T(const lbch_handle* h)
+{
+    return h->timed && h->t_row >= 0 ? h->d_T + (size_t)h->t_row * h->n_inst : nullptr;
+}
+inline int launch_reads_n(const lbch_handle* h) { return h->model3 || (h->timed && h->t_row < 0); }
 
 // The row sweep keeps the populations unless every instance has tau_g = 1 (and no test asks for them).
 inline bool sweep_gen(const lbch_handle* h) { return !h->tau1 || h->force_general; }

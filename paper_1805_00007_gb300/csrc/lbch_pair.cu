@@ -27,6 +27,8 @@ cudaError_t launch_pair_v(lbch_handle* h, int parity)
     a.t_off = h->t_off;
     a.t_adv = h->t_adv;
     a.need_time = h->need_time;
+    a.Tf = launch_T(h);
+    a.read_n = launch_reads_n(h);
     a.debug_skip = h->debug_skip;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ps.grid);

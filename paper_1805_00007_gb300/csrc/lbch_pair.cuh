@@ -36,6 +36,8 @@ struct PairArgs {
     int t_off;              // the launch's first step is ctl->time + t_off, its second one step later
     int t_adv;              // when nonzero, the launch's last CTA advances ctl->time by t_adv
     int need_time;          // some instance's flow depends on the step index
+    int read_n;             // ... and the launch reads it (no table of time factors)
+    const double* Tf;       // the instances' time factors at the first step, then at the second, or null (step_T)
     int debug_skip;         // test hook: CTA 0 never issues its first table copy (its bounded wait runs out)
 };
 
@@ -380,9 +382,9 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __
         if (any) ld.load(S, a.phi_in + rb, a.lo_in + rb);
         if (tid == 0) {
             if (any) wait_tables();
-            s_time = a.need_time ? a.ctl->time : 0;
-            s_T[0] = (C)vel_t(I.vel, I.Tper, s_time + a.t_off);
-            s_T[1] = (C)vel_t(I.vel, I.Tper, s_time + a.t_off + 1);
+            s_time = a.read_n ? a.ctl->time : 0;
+            s_T[0] = (C)step_T(a.Tf, 0, I, s_time + a.t_off);
+            s_T[1] = (C)step_T(a.Tf, 1, I, s_time + a.t_off + 1);
         }
         __syncthreads();
         n = s_time + a.t_off;
@@ -425,10 +427,10 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __
         if (any) ld.load(S, a.phi_in + rb, a.lo_in + rb);
         if (tid == 0) {
             if (any) wait_tables();
-            s_time = a.need_time ? a.ctl->time : 0;
+            s_time = a.read_n ? a.ctl->time : 0;
             if (s_k >= 0) {
-                s_T[0] = (C)vel_t(s_I.vel, s_I.Tper, s_time + a.t_off);
-                s_T[1] = (C)vel_t(s_I.vel, s_I.Tper, s_time + a.t_off + 1);
+                s_T[0] = (C)step_T(a.Tf, s_k, s_I, s_time + a.t_off);
+                s_T[1] = (C)step_T(a.Tf, a.n_inst + s_k, s_I, s_time + a.t_off + 1);
             }
         }
         __syncthreads();
@@ -439,8 +441,8 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __
                 if (tid == 0) {
                     pair_fetch_tables<C, P, TX, TY>(S, a.ttabs, t, &s_tbar);
                     if (locate(t)) {
-                        s_T[0] = (C)vel_t(s_I.vel, s_I.Tper, n);
-                        s_T[1] = (C)vel_t(s_I.vel, s_I.Tper, n + 1);
+                        s_T[0] = (C)step_T(a.Tf, s_k, s_I, n);
+                        s_T[1] = (C)step_T(a.Tf, a.n_inst + s_k, s_I, n + 1);
                     }
                 }
                 __syncthreads();
@@ -460,7 +462,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __
         unsigned int prev = atomicAdd(&a.ctl->done, 1u);
         if (prev == gridDim.x - 1) {
             a.ctl->done = 0u;
-            a.ctl->time = (a.need_time ? n - a.t_off : a.ctl->time) + a.t_adv;
+            a.ctl->time = (a.read_n ? n - a.t_off : a.ctl->time) + a.t_adv;
         }
     }
 }

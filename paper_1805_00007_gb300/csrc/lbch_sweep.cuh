@@ -54,7 +54,8 @@ struct SweepArgs {
     Ctl* ctl;
     int t_off;              // this launch's step is ctl->time + t_off
     int t_adv;              // when nonzero, the launch's last CTA advances ctl->time by t_adv
-    int need_time;          // some instance needs the step index (a time-dependent flow)
+    int read_n;             // the launch reads the step index: Model III, or a time factor without a table
+    const double* Tf;       // the instances' time factors at this launch's step, or null (step_T)
     S* g_out;               // populations (GEN): g[(row * nq + plane) * pitch + column]
     int rows;               // stored rows of the population arrays
     const C* H_in;          // M3 (Model III): H(t - 1) of Eq. F2-1's time derivatives, two planes (x, y) of
@@ -295,9 +296,9 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
             const int t = blockIdx.x + j * stride;
             if (t < a.total_tiles && !(a.debug_skip && blockIdx.x == 0 && j == 0)) issue(t, j);
         }
-        // the counter is read only when a flow depends on time; otherwise nothing waits on that load
-        s_time = a.need_time ? a.ctl->time : 0;
-        if (s_tile_inst >= 0) s_T = (C)vel_t(s_I.vel, s_I.Tper, s_time + a.t_off);
+        // the counter is read only when the launch needs the step index; otherwise nothing waits on that load
+        s_time = a.read_n ? a.ctl->time : 0;
+        if (s_tile_inst >= 0) s_T = (C)step_T(a.Tf, s_tile_inst, s_I, s_time + a.t_off);
     }
     __syncthreads();
     // (the step index stays in shared memory: s_time + a.t_off, read where an instance changes and at exit,
@@ -767,7 +768,7 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
             __syncthreads();
             if (tid == 0) {
                 s_tile_inst = k_t;
-                s_T = (C)vel_t(s_I.vel, s_I.Tper, s_time + a.t_off);
+                s_T = (C)step_T(a.Tf, k_t, s_I, s_time + a.t_off);
             }
         }
         __syncthreads();
@@ -802,7 +803,7 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(C) == 8 ? 8 : 12) / NW)
         const unsigned int prev = atomicAdd(&a.ctl->done, 1u);
         if (prev == gridDim.x - 1) {
             a.ctl->done = 0u;
-            a.ctl->time = (a.need_time ? s_time : a.ctl->time) + a.t_adv;
+            a.ctl->time = (a.read_n ? s_time : a.ctl->time) + a.t_adv;
         }
     }
 }

@@ -26,7 +26,8 @@ cudaError_t launch_sweep_v(lbch_handle* h, int parity)
     a.ctl = h->ctl;
     a.t_off = h->t_off;
     a.t_adv = h->t_adv;
-    a.need_time = h->need_time;
+    a.Tf = launch_T(h);
+    a.read_n = launch_reads_n(h);
     a.g_out = static_cast<S*>(h->g[parity ^ 1]);
     a.rows = h->rows;
     a.H_in = M3 ? static_cast<const C*>(h->H[parity]) : nullptr;
