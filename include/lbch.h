@@ -206,7 +206,8 @@ lbch_status lb_ch_info(lbch_handle* h, double* out);
  * the populations, 3 = the coupled Navier-Stokes kernels, 4 = tile kernel without the populations, 5 = the
  * two-step kernel: two steps per launch, periodic instances with tau_g = 1),
  * out[1] = the shape index in use (see
- * lb_ch_tune), out[2] x out[3] = output nodes of one tile, out[4] = output rows per warp of the row
+ * lb_ch_tune), out[2] x out[3] = output nodes of one tile (of the row sweep: the nominal tile its configuration is
+ * named by), out[4] = output rows per warp of the row
  * sweep (0 otherwise), out[5] = threads per thread block.  out must hold 6 ints. */
 lbch_status lb_ch_kernel_info(lbch_handle* h, int* out);
 
@@ -214,7 +215,8 @@ lbch_status lb_ch_kernel_info(lbch_handle* h, int* out);
 void* lb_ch_stream(lbch_handle* h);
 
 /* Kernel and tile-shape autotuner.  The step has three kernel forms, each built for several shapes: the
- * row sweep (warps sweeping 56-column strips; tiles of 56 x 48, 56 x 24 and twice 56 x 12 output nodes),
+ * row sweep (warps sweeping strips of 56 or 58 columns, the grid cut into as many as 16, 8, 4 or 12 warps per SM --
+ * fewer where its registers allow fewer --; reported as tiles of 56 x 48, 56 x 24, 56 x 12 and 56 x 24 output nodes),
  * the tile kernel (each tile's stencil fields staged in shared memory; 32x16, 32x8 and 16x8 with 256
  * threads and 32x16 with 768 on the float paths; 32x8 and 16x8 with 256 and 32x8 with 512 for LBCH_F64)
  * and, for handles whose instances are all periodic with tau_g = 1 in LBCH_F32 or LBCH_F64, the two-step
@@ -269,7 +271,8 @@ lbch_status lb_ch_step_taped(lbch_handle* h, long nsteps, void* tape);
 lbch_status lb_ch_adjoint_sweep(lbch_handle* h, const void* tape, long n0, long nsteps);
 
 /* Test hook for the failure path of the step kernel's bounded waits.  With hook
- * LBCH_HOOK_SKIP_FIRST_LOAD and value != 0, the next step launches run without CUDA graphs and their
+ * LBCH_HOOK_SKIP_FIRST_LOAD and value != 0, the next step launches run without CUDA graphs, on the tile kernel
+ * where the handle would step with the row sweep (which has no such wait), and their
  * first thread block never issues its first tile copy, so its bounded wait runs out (after about a
  * second); the kernel then returns cleanly and the next lb_ch_observe reports LBCH_ETIMEOUT.  The
  * handle's state is not advanced correctly afterwards and should be freed.  With hook

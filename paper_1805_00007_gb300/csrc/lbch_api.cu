@@ -10,6 +10,7 @@
 #include "lbch_internal.h"
 #include "lbch_kernels.cuh"
 #include "lbch_ns.cuh"
+#include "lbch_sweep.cuh"
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -219,20 +220,20 @@ cudaError_t launch_step_t(lbch_handle* h, int parity)
 // two-step kernel is selected (and applies), it takes the steps two at a time and the one-step kernel
 // takes an odd last step.
 inline bool use_pair(const lbch_handle* h) { return h->pair && pair_ok(h); }
-inline bool use_sweep(const lbch_handle* h) { return !h->force_tile && !h->coupled; }
+// (the sweep has no bounded wait to run out: with the test hook that withholds a copy, the tile kernel steps instead)
+inline bool use_sweep(const lbch_handle* h) { return !h->force_tile && !h->coupled && !h->debug_skip; }
 // sweep configurations built for the handle (those with Model III: the two unrolled ones)
 inline int n_sweep_shapes(const lbch_handle* h) { return h->model3 ? kM3SweepShapes : kSweepShapes; }
 inline int n_active(const lbch_handle* h)
 {
     return h->coupled ? 1 : (use_pair(h) ? kPairShapes : (use_sweep(h) ? n_sweep_shapes(h) : n_shapes(h->prec)));
 }
-inline const lbch_handle::PerShape& active_ps(const lbch_handle* h)
-{
-    return use_pair(h) ? h->pr[h->pshape] : (use_sweep(h) ? h->sw[h->shape] : h->ps[h->shape]);
-}
 inline int active_grid(const lbch_handle* h)
 {
-    return !use_pair(h) && use_sweep(h) && sweep_gen(h) ? h->sw[h->shape].grid_gen : active_ps(h).grid;
+    if (use_pair(h)) return h->pr[h->pshape].grid;
+    if (!use_sweep(h)) return h->ps[h->shape].grid;
+    const lbch_handle::SweepCut& sc = h->sw[h->shape][sweep_gen(h)];
+    return (sc.n_items + sc.nw - 1) / sc.nw;
 }
 inline Shape active_tile(const lbch_handle* h)
 {
@@ -264,21 +265,46 @@ cudaError_t launch_sweep(lbch_handle* h, int parity)
     }
 }
 
-cudaError_t prepare_sweep(lbch_handle* h, int k)
+cudaError_t prepare_sweep(lbch_handle* h, bool gen, SweepFit* fit)
 {
-    if (h->model3 && k < kM3SweepShapes) {
+    if (h->model3) {
         switch (h->prec) {
-        case LBCH_F64: return lbch_prepare_sweep_f64_m3(h, k);
-        case LBCH_F32: return lbch_prepare_sweep_f32_m3(h, k);
-        default: return lbch_prepare_sweep_f16s_m3(h, k);
+        case LBCH_F64: return lbch_prepare_sweep_f64_m3(h, gen, fit);
+        case LBCH_F32: return lbch_prepare_sweep_f32_m3(h, gen, fit);
+        default: return lbch_prepare_sweep_f16s_m3(h, gen, fit);
         }
     }
     switch (h->prec) {
-    case LBCH_F64: return lbch_prepare_sweep_f64(h, k);
-    case LBCH_F32: return lbch_prepare_sweep_f32(h, k);
-    default: return lbch_prepare_sweep_f16s(h, k);
+    case LBCH_F64: return lbch_prepare_sweep_f64(h, gen, fit);
+    case LBCH_F32: return lbch_prepare_sweep_f32(h, gen, fit);
+    default: return lbch_prepare_sweep_f16s(h, gen, fit);
     }
 }
+
+// Rows per strip of the row sweep, for strips of `width` columns over the handle's instances shared out among `warps`
+// resident warps: the length that takes the fewest row steps, a strip of R rows taking R + 6 of them and the strips
+// coming in rounds of `warps` (one round, where the grid allows strips that long).
+int sweep_rows(const lbch_handle* h, const SweepFit& fit, int warps)
+{
+    int most = 1, best = 1;
+    for (const InstDev& d : h->inst) most = std::max(most, d.ny);
+    long long best_cost = -1;
+    for (int R = 1; R <= most; R += std::max(1, R / 32)) {
+        long long items = 0;
+        for (const InstDev& d : h->inst)
+            items += (long long)((d.nx + fit.lead + fit.width - 1) / fit.width) * ((d.ny + R - 1) / R);
+        const long long cost = (items + warps - 1) / warps * (R + 6);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = R;
+        }
+    }
+    return best;
+}
+
+// Cut the handle's grids into the strips of configuration k (gen: of the form with the populations), side by side and
+// row block after row block of one instance after the other, so that neighbouring strips go to one block's warps.
+cudaError_t cut_sweep(lbch_handle* h, int k, bool gen, const SweepFit& fit);
 
 // Dynamic shared memory of the step kernel, and the persistent grid that fits the device, for shape k.
 template <typename C, typename S, typename P, int TX, int TY, int NTT = NT>
@@ -666,6 +692,45 @@ void stage_give(double* p, size_t bytes)
     cudaFreeHost(p);
 }
 
+// Warps per block for n strips: on a grid that fills the device, blocks as large as an SM takes keep the SM's warps on
+// neighbouring strips of the same rows, and so on few pages and DRAM rows (4096^2, us per step in blocks of 2, 8 and 16
+// warps: half storage with the populations 187, 184, 175; float at tau_g = 1 119, 118, 116); smaller grids want their
+// strips on as many SMs as there are (100^2: 3.4 us in blocks of two, 5.2 in blocks of 16).
+int sweep_block(const SweepFit& fit, long long n)
+{
+    int nw = 2;
+    while (nw < fit.nw && 2 * n >= 3LL * nw * fit.sms) nw *= 2;
+    return nw;
+}
+
+cudaError_t cut_sweep(lbch_handle* h, int k, bool gen, const SweepFit& fit)
+{
+    lbch_handle::SweepCut& sc = h->sw[k][gen];
+    const int R = sweep_rows(h, fit, std::min(kSweepWarps[k], fit.warps) * fit.sms);
+    std::vector<SweepItem> items;
+    sc.rows_per = 0;
+    for (int i = 0; i < h->n_inst; i++) {
+        const InstDev& d = h->inst[i];
+        const int strips = (d.nx + fit.lead + fit.width - 1) / fit.width;
+        const int blocks = (d.ny + R - 1) / R, rows = (d.ny + blocks - 1) / blocks;  // of nearly equal length
+        sc.rows_per = std::max(sc.rows_per, rows);
+        if (h->n_inst == 1) {
+            sc.strips = strips;
+            sc.n_items = strips * ((d.ny + rows - 1) / rows);
+            sc.nw = sweep_block(fit, sc.n_items);
+            return cudaSuccess;
+        }
+        for (int y = 0; y < d.ny; y += rows)
+            for (int c = 0; c < strips; c++) items.push_back({i, c * fit.width, y, std::min(rows, d.ny - y)});
+    }
+    sc.n_items = (int)items.size();
+    sc.nw = sweep_block(fit, sc.n_items);
+    cudaError_t e = dalloc(h, &sc.d_items, sizeof(SweepItem) * items.size());
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(sc.d_items, items.data(), sizeof(SweepItem) * items.size(), cudaMemcpyHostToDevice, h->stream);
+    return e;
+}
+
 void release(lbch_handle* h)
 {
     for (int k = 0; k < 2; k++) {
@@ -680,10 +745,8 @@ void release(lbch_handle* h)
     dfree(h, h->d_inst);
     dfree(h, h->d_tabs_f);
     for (int k = 0; k < kMaxShapes; k++) dfree(h, h->ps[k].d_tile_begin);
-    for (int k = 0; k < kSweepShapes; k++) {
-        dfree(h, h->sw[k].d_tile_begin);
-        dfree(h, h->sw[k].d_tiles);
-    }
+    for (int k = 0; k < kSweepShapes; k++)
+        for (int gen = 0; gen < 2; gen++) dfree(h, h->sw[k][gen].d_items);
     for (int k = 0; k < kPairShapes; k++) {
         dfree(h, h->pr[k].d_tile_begin);
         dfree(h, h->pr[k].d_ttabs);
@@ -745,69 +808,6 @@ lbch_status encode_maps(lbch_handle* h, int sk)
             if (r != CUDA_SUCCESS) return fail(LBCH_ECUDA, "tensor map of phi (low part): CUresult %d", (int)r);
         } else {
             ps.tm_lo[k] = ps.tm_phi[k];  // unused by the kernels without a low part
-        }
-    }
-    return LBCH_OK;
-}
-
-// The row-sweep kernel's boxes: phi over 64 columns and the tile's rows plus three halo rows on each
-// side; the low part of phi over the output rows.
-lbch_status encode_sweep_maps(lbch_handle* h, int sk)
-{
-    const Shape sh = sweep_tile(sk);
-    lbch_handle::PerShape& ps = h->sw[sk];
-    EncodeTiledFn enc = encode_fn();
-    if (!enc) return fail(LBCH_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    CUtensorMapDataType pt = h->phi_elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-    cuuint32_t es[2] = {1, 1};
-    cuuint64_t pdim[2] = {(cuuint64_t)h->pitch, (cuuint64_t)h->rows};
-    for (int k = 0; k < 2; k++) {
-        cuuint64_t pstr[1] = {(cuuint64_t)h->pitch * h->phi_elem};
-        cuuint32_t pbox[2] = {64u, (cuuint32_t)(sh.ty + 6)};
-        CUresult r = enc(&ps.tm_phi[k], pt, 2, h->phi[k], pdim, pstr, pbox, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                         CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(LBCH_ECUDA, "tensor map of phi (row sweep): CUresult %d", (int)r);
-        if (h->lo[k]) {
-            cuuint64_t lstr[1] = {(cuuint64_t)h->pitch * 4};
-            cuuint32_t lbox[2] = {64u, (cuuint32_t)sh.ty};
-            r = enc(&ps.tm_lo[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->lo[k], pdim, lstr, lbox, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (r != CUDA_SUCCESS) return fail(LBCH_ECUDA, "tensor map of phi, low part (row sweep): CUresult %d", (int)r);
-        } else {
-            ps.tm_lo[k] = ps.tm_phi[k];  // unused without a low part
-        }
-        ps.tm_g[k] = ps.tm_phi[k];
-    }
-    return LBCH_OK;
-}
-
-// The row sweep's ring fills: one row of the population planes (64 columns x nq planes), and one row of
-// the low part of phi.
-lbch_status encode_row_maps(lbch_handle* h)
-{
-    EncodeTiledFn enc = encode_fn();
-    if (!enc) return fail(LBCH_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    CUtensorMapDataType gt = h->prec == LBCH_F64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64
-                           : (h->prec == LBCH_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16);
-    for (int k = 0; k < 2; k++) {
-        cuuint64_t gdim[3] = {(cuuint64_t)h->pitch, (cuuint64_t)h->nq, (cuuint64_t)h->rows};
-        cuuint64_t gstr[2] = {(cuuint64_t)h->pitch * h->g_elem, (cuuint64_t)h->pitch * h->g_elem * h->nq};
-        cuuint32_t gbox[3] = {64u, (cuuint32_t)h->nq, 1u};
-        cuuint32_t es[3] = {1, 1, 1};
-        CUresult r = enc(&h->tm_grow[k], gt, 3, h->g[k], gdim, gstr, gbox, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                         CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(LBCH_ECUDA, "tensor map of a population row: CUresult %d", (int)r);
-        if (h->lo[k]) {
-            cuuint64_t ldim[2] = {(cuuint64_t)h->pitch, (cuuint64_t)h->rows};
-            cuuint64_t lstr[1] = {(cuuint64_t)h->pitch * 4};
-            cuuint32_t lbox[2] = {64u, 1u};
-            r = enc(&h->tm_lorow[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->lo[k], ldim, lstr, lbox, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (r != CUDA_SUCCESS) return fail(LBCH_ECUDA, "tensor map of a row of phi's low part: CUresult %d", (int)r);
-        } else {
-            h->tm_lorow[k] = h->tm_grow[k];  // unused without a low part
         }
     }
     return LBCH_OK;
@@ -1117,17 +1117,6 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
         tile_begin[sk].push_back(t);
         h->ps[sk].total_tiles = t;
     }
-    std::vector<int> sweep_begin[kSweepShapes];
-    for (int sk = 0; sk < kSweepShapes; sk++) {
-        const Shape sh = sweep_tile(sk);
-        int t = 0;
-        for (int k = 0; k < n_inst; k++) {
-            sweep_begin[sk].push_back(t);
-            t += ((params[k].nx + sh.tx - 1) / sh.tx) * ((params[k].ny + sh.ty - 1) / sh.ty);
-        }
-        sweep_begin[sk].push_back(t);
-        h->sw[sk].total_tiles = t;
-    }
     std::vector<int> pair_begin[kPairShapes];
     for (int sk = 0; sk < kPairShapes; sk++) {
         const Shape sh = pair_shape(prec, sk);
@@ -1170,28 +1159,10 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
                             cudaMemcpyHostToDevice, h->stream));
     }
     if (!coupled) {
-        for (int sk = 0; sk < kSweepShapes; sk++) {
-            CKI(prepare_sweep(h, sk));
-            CKI(dalloc(h, &h->sw[sk].d_tile_begin, sizeof(int) * (n_inst + 1)));
-            CKI(cudaMemcpyAsync(h->sw[sk].d_tile_begin, sweep_begin[sk].data(), sizeof(int) * (n_inst + 1),
-                                cudaMemcpyHostToDevice, h->stream));
-            // the tiles of every instance, those that need the wall body (their collision rows or the rows
-            // their stencils read come within two rows of a wall) after all the others
-            const Shape sh = sweep_tile(sk);
-            std::vector<int4> inner, edge;
-            for (int k = 0; k < n_inst; k++) {
-                const lbch_params& p = params[k];
-                const int tiles_x = (p.nx + sh.tx - 1) / sh.tx, tiles_y = (p.ny + sh.ty - 1) / sh.ty;
-                for (int l = 0; l < tiles_x * tiles_y; l++) {
-                    const int x0 = (l % tiles_x) * sh.tx, y0 = (l / tiles_x) * sh.ty;
-                    const bool w = p.walls && (y0 < 2 || y0 + sh.ty + 1 > p.ny - 1);
-                    (w ? edge : inner).push_back(make_int4(k, x0, y0, w ? 1 : 0));
-                }
-            }
-            inner.insert(inner.end(), edge.begin(), edge.end());
-            CKI(dalloc(h, &h->sw[sk].d_tiles, sizeof(int4) * inner.size()));
-            CKI(cudaMemcpyAsync(h->sw[sk].d_tiles, inner.data(), sizeof(int4) * inner.size(), cudaMemcpyHostToDevice,
-                                h->stream));
+        for (int gen = h->tau1 ? 0 : 1; gen < 2; gen++) {  // (with tau_g = 1 the populations are kept for tests only)
+            SweepFit fit;
+            CKI(prepare_sweep(h, gen, &fit));
+            for (int sk = 0; sk < kSweepShapes; sk++) CKI(cut_sweep(h, sk, gen, fit));
         }
         for (int sk = 0; sk < kPairShapes && prec != LBCH_F16S; sk++) {
             CKI(lbch_prepare_pair(h, sk));
@@ -1240,10 +1211,11 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     const size_t cells = (size_t)h->rows * h->pitch;
     const size_t gbytes = cells * h->nq * h->g_elem;
     const size_t pbytes = cells * h->phi_elem;
+    const size_t spare = 3 * (size_t)h->pitch;  // the row sweep reads phi up to three rows past its last
     for (int k = 0; k < 2; k++) {
         CKI(dalloc(h, &h->g[k], gbytes));
-        CKI(dalloc(h, &h->phi[k], pbytes));
-        if (prec == LBCH_F32) CKI(dalloc(h, &h->lo[k], cells * sizeof(float)));
+        CKI(dalloc(h, &h->phi[k], pbytes + spare * h->phi_elem));
+        if (prec == LBCH_F32) CKI(dalloc(h, &h->lo[k], (cells + spare) * sizeof(float)));
         if (h->model3) CKI(dalloc(h, &h->H[k], 2 * cells * h->c_elem()));
     }
     CKI(dalloc(h, &h->phi0, cells * sizeof(double)));
@@ -1261,8 +1233,6 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     CKI(dalloc(h, &h->result, sizeof(double) * RED_NV * (size_t)n_inst));
     lbch_status st = LBCH_OK;
     for (int sk = 0; sk < n_shapes(prec) && st == LBCH_OK; sk++) st = encode_maps(h, sk);
-    for (int sk = 0; !coupled && sk < kSweepShapes && st == LBCH_OK; sk++) st = encode_sweep_maps(h, sk);
-    if (!coupled && st == LBCH_OK) st = encode_row_maps(h);
     if (st != LBCH_OK) return bail(st);
 
     // the initial field in the padded layout, ghost frame included, through pinned staging
@@ -1429,10 +1399,10 @@ lbch_status lb_ch_step(lbch_handle* h, long nsteps)
             h->n += chunk;
             nsteps -= chunk;
         } else {
-            // a few last steps form their time factors themselves: the table's own launch costs about as much as
-            // the factors of three launches
+            // a few last steps of the kernels with one block per SM form their time factors themselves: the table's own
+            // launch costs about as much as the factors of three launches (in the row sweep every warp would)
             const int per = two && nsteps >= 2 ? 2 : 1;
-            if (row + per > rows && h->timed && nsteps > 3 * per) {
+            if (row + per > rows && h->timed && (nsteps > 3 * per || (per == 1 && use_sweep(h)))) {
                 rows = (int)std::min<long>(nsteps, kTimeSteps);
                 row = 0;
                 CK(time_table(h, rows));
@@ -1603,8 +1573,8 @@ lbch_status lb_ch_kernel_info(lbch_handle* h, int* out)
     out[1] = pr ? h->pshape : h->shape;
     out[2] = sh.tx;
     out[3] = sh.ty;
-    out[4] = sw && !pr ? kSweep[h->shape].ty : 0;
-    out[5] = h->coupled ? 256 : sh.nt;
+    out[4] = sw && !pr ? h->sw[h->shape][sweep_gen(h)].rows_per : 0;
+    out[5] = h->coupled ? 256 : sw && !pr ? 32 * h->sw[h->shape][sweep_gen(h)].nw : sh.nt;
     return LBCH_OK;
 }
 
@@ -1753,8 +1723,12 @@ lbch_status lb_ch_step_taped(lbch_handle* h, long nsteps, void* tape)
         return LBCH_OK;
     }
     for (long k = 0; k < nsteps; k++) {
+        if (k % kTimeSteps == 0) CK(time_table(h, (int)std::min<long>(nsteps - k, kTimeSteps)));
         CK(tape_launch(h, cur_buf(h), t + (size_t)k * stride));
-        CK(launch_step(h, cur_buf(h)));  // a one-step launch (the two-step kernel would skip a tape entry)
+        h->t_row = (int)(k % kTimeSteps);
+        const cudaError_t e = launch_step(h, cur_buf(h));  // a one-step launch (the two-step kernel would skip a tape entry)
+        h->t_row = -1;
+        CK(e);
         h->n += 1;
     }
     return LBCH_OK;

@@ -10,14 +10,19 @@
 constexpr int kMaxShapes = 5;
 struct Shape { int tx, ty, nt; };  // output nodes of a tile, threads per block
 
-// Configurations of the row-sweep kernel (tau_g = 1): TY output rows per warp, NW warps per CTA; a tile
-// is 56 columns by NW TY rows.  lb_ch_tune picks among them as among the tile shapes.
-struct SweepCfg { int ty, nw; bool compact; };
-constexpr SweepCfg kSweep[4] = {{12, 4, false}, {6, 4, false}, {6, 2, true}, {3, 4, true}};
+// Configurations of the row-sweep kernel: the warps per SM among which the grid is cut into strips (fewer where the
+// kernel's registers allow fewer).  Many warps hide latency and give long runs of rows on large grids; a grid whose
+// strips would get only a few rows each steps faster with fewer, longer ones (lb_ch_tune; sweep_cost).  A
+// configuration is reported under a nominal tile of 56 columns.
 constexpr int kSweepShapes = 4;
-constexpr int kM3SweepShapes = 2;  // configurations built for handles with a Model III instance
+constexpr int kM3SweepShapes = 2;  // configurations used for handles with a Model III instance
+constexpr int kSweepWarps[kSweepShapes] = {16, 8, 4, 12};
+constexpr int kSweepTileRows[kSweepShapes] = {48, 24, 12, 24};
 constexpr int kSweepW = 56;
-inline Shape sweep_tile(int k) { return Shape{kSweepW, kSweep[k].ty * kSweep[k].nw, 32 * kSweep[k].nw}; }
+inline Shape sweep_tile(int k) { return Shape{kSweepW, kSweepTileRows[k], 0}; }
+// What a sweep kernel allows on the device: warps resident per SM, SMs, and the columns of its strips.
+// (and of one block).
+struct SweepFit { int warps, sms, nw, width, lead; };
 
 // Tile shapes of the two-step kernel (periodic instances, tau_g = 1; f32 and f64 only).
 constexpr int kPairShapes = 4;
@@ -60,15 +65,17 @@ struct lbch_handle {
     struct PerShape {           // what depends on the tile shape
         int total_tiles = 0;
         int grid = 0;           // persistent CTAs per step launch
-        int grid_gen = 0;       // row sweep with the populations (the tile kernel uses grid)
         int* d_tile_begin = nullptr;
-        int4* d_tiles = nullptr;  // row-sweep configurations: each tile's (instance, x0, y0, wall body needed),
-                                  // interior tiles first (see lbch_sweep.cuh)
         void* d_ttabs = nullptr;  // two-step shapes: each tile's velocity tables, contiguous (see lbch_pair.cuh)
         CUtensorMap tm_g[2], tm_phi[2], tm_lo[2];
-    } ps[kMaxShapes], sw[kSweepShapes], pr[kPairShapes];  // tile kernel shapes; row-sweep configurations
-                                                          // (tm_g unused); two-step shapes (no maps)
-    CUtensorMap tm_grow[2], tm_lorow[2];  // one row of the populations / of phi's low part (row sweep)
+    } ps[kMaxShapes], pr[kPairShapes];  // tile kernel shapes; two-step shapes (no maps)
+    struct SweepCut {           // a row-sweep configuration's division of the handle's grids (see lbch_sweep.cuh)
+        int n_items = 0;        // strips, one per warp
+        int strips = 0;         // a single instance's strips side by side
+        int rows_per = 0;       // rows of one strip (the most, over several instances)
+        int nw = 2;             // warps per block
+        void* d_items = nullptr;  // several instances: every strip (SweepItem)
+    } sw[kSweepShapes][2];      // [..][0] without the populations (tau_g = 1), [..][1] with them
     void* g[2] = {nullptr, nullptr};
     void* phi[2] = {nullptr, nullptr};
     float* lo[2] = {nullptr, nullptr};  // low part of phi (float path)
@@ -135,16 +142,16 @@ inline bool pair_ok(const lbch_handle* h)
 LBCH_INTERNAL cudaError_t lbch_launch_sweep_f64(lbch_handle* h, int parity);
 LBCH_INTERNAL cudaError_t lbch_launch_sweep_f32(lbch_handle* h, int parity);
 LBCH_INTERNAL cudaError_t lbch_launch_sweep_f16s(lbch_handle* h, int parity);
-LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f64(lbch_handle* h, int k);
-LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f32(lbch_handle* h, int k);
-LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f16s(lbch_handle* h, int k);
-// The same for handles with a Model III instance (lbch_sweep_*_m3.cu; configurations 0 and 1).
+LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f64(lbch_handle* h, bool gen, SweepFit* fit);
+LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f32(lbch_handle* h, bool gen, SweepFit* fit);
+LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f16s(lbch_handle* h, bool gen, SweepFit* fit);
+// The same for handles with a Model III instance (lbch_sweep_*_m3.cu).
 LBCH_INTERNAL cudaError_t lbch_launch_sweep_f64_m3(lbch_handle* h, int parity);
 LBCH_INTERNAL cudaError_t lbch_launch_sweep_f32_m3(lbch_handle* h, int parity);
 LBCH_INTERNAL cudaError_t lbch_launch_sweep_f16s_m3(lbch_handle* h, int parity);
-LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f64_m3(lbch_handle* h, int k);
-LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f32_m3(lbch_handle* h, int k);
-LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f16s_m3(lbch_handle* h, int k);
+LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f64_m3(lbch_handle* h, bool gen, SweepFit* fit);
+LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f32_m3(lbch_handle* h, bool gen, SweepFit* fit);
+LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f16s_m3(lbch_handle* h, bool gen, SweepFit* fit);
 // Two-step launches and set-up (lbch_pair.cu); pshape names a pair_shape().
 LBCH_INTERNAL cudaError_t lbch_launch_pair(lbch_handle* h, int parity);
 LBCH_INTERNAL cudaError_t lbch_prepare_pair(lbch_handle* h, int k);

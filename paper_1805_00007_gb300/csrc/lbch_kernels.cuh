@@ -294,8 +294,14 @@ __device__ __forceinline__ void node_force(C ph, C gmx, C gmy, C gDx, C gDy, C P
                                            const Consts<C>& K0, C& Jx, C& Jy)
 {
     const C fct = op_mul(op_mul(ph, ph), node_rcp(op_fma(K0.ra, ph, K0.rb)));
-    Jx = op_fma(fct, gmx, model2 ? op_fma(K0.Kd, gDx, Px) : Px);
-    Jy = op_fma(fct, gmy, model2 ? op_fma(K0.Kd, gDy, Py) : Py);
+    Jx = Px;
+    Jy = Py;
+    if (model2) {
+        Jx = op_fma(K0.Kd, gDx, Jx);
+        Jy = op_fma(K0.Kd, gDy, Jy);
+    }
+    Jx = op_fma(fct, gmx, Jx);
+    Jy = op_fma(fct, gmy, Jy);
 }
 
 // Model III: the complete diffusive-scale force of Eq. F2-1, with the time derivatives on the convective
@@ -359,7 +365,10 @@ __device__ __forceinline__ C bounce(C post_opp, C ph, C uwx, C uwy)
     const C cuw = cx(q) == 0 ? (cy(q) > 0 ? uwy : -uwy)
                 : (cy(q) == 0 ? (cx(q) > 0 ? uwx : -uwx)
                 : (cx(q) > 0 ? (cy(q) > 0 ? uwx + uwy : uwx - uwy) : (cy(q) > 0 ? uwy - uwx : -(uwx + uwy))));
-    return op_fma(op_mul(C(6) * wq<C>(q), ph), cuw, post_opp);
+    const C g = op_fma(op_mul(C(6) * wq<C>(q), ph), cuw, post_opp);
+    // 2 and 4 pass through a quarter, as which the sums at tau_g = 1 carry them: the same bits in every form, down to
+    // the smallest numbers
+    return q == 2 || q == 4 ? op_mul(C(4), op_mul(C(0.25), g)) : g;
 }
 
 // Sum of the streamed populations g_1..g_8(t+1) at a node, grouped by the column they come from: the

@@ -7,7 +7,7 @@ cudaError_t lbch_launch_sweep_f64_m3(lbch_handle* h, int parity)
     return lbch::launch_sweep_t<double, double, double, false, true>(h, parity);
 }
 
-cudaError_t lbch_prepare_sweep_f64_m3(lbch_handle* h, int k)
+cudaError_t lbch_prepare_sweep_f64_m3(lbch_handle* h, bool gen, SweepFit* fit)
 {
-    return lbch::prepare_sweep_t<double, double, double, false, true>(h, k);
+    return lbch::prepare_sweep_t<double, double, double, false, true>(h, gen, fit);
 }
