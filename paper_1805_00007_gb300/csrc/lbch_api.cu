@@ -74,14 +74,14 @@ static_assert(kGraphChunk % 4 == 0 && kGraphBig % kGraphChunk == 0, "graph sizes
 // times them on the handle's own problem and keeps the fastest; the first one is the default.  Every
 // TX divides 32 and every TY divides 16, so one storage layout serves all shapes.
 constexpr int NT = 256;
-// FP64 32 x 16 with 736 threads: 128 tiles at 256^2, at most one per SM, and the least recomputed halo of
-// the shapes that fit that count (the FP64 step is bound by the FP64 pipe, so the halo's share counts);
-// 736 threads take each phase in one pass (0.3 to 0.7 % faster than 512 at 1024^2 to 4096^2).
-// FP64 32 x 14 with 672 threads: 152 tiles at 256^2, one per SM, with a little less halo per SM than
-// 32 x 16; 672 threads take every phase in one pass (mu and D on the tile + 2 are 648 nodes; with 576
-// threads a second pass of three warps left the FP64 pipe short: 25.2 against 24.65 us per step).  (Only for FP64: its per-tile copy of
+// FP64 32 x 16 with 768 threads: 128 tiles at 256^2, at most one per SM, and the least recomputed halo of
+// the shapes that fit that count (the FP64 step is bound by the FP64 pipe, so the halo's share counts).
+// FP64 32 x 14 with 704 threads: 152 tiles at 256^2, one per SM, with a little less halo per SM than
+// 32 x 16.  Both thread counts take every phase in one pass (the widest has 38 x 20 and 38 x 18 nodes; with 736 and
+// 672 threads, us per step: 2048^2 901 and 923 against 879 and 894, 256^2 18.2 and 16.4 against 17.8 and 16.0).  (32 x 14
+// only for FP64: its per-tile copy of
 // the Y tables starts at row y0, which is 16-byte aligned for 8-byte entries and even y0 only.)
-constexpr Shape kShapes64[5] = {{32, 8, 256}, {16, 8, 256}, {32, 8, 512}, {32, 16, 736}, {32, 14, 672}};
+constexpr Shape kShapes64[5] = {{32, 8, 256}, {16, 8, 256}, {32, 8, 512}, {32, 16, 768}, {32, 14, 704}};
 constexpr Shape kShapesF[4] = {{32, 16, 256}, {32, 8, 256}, {16, 8, 256}, {32, 16, 768}};
 inline int n_shapes(int prec) { return prec == LBCH_F64 ? 5 : 4; }
 inline Shape shape_of(int prec, int k) { return prec == LBCH_F64 ? kShapes64[k] : kShapesF[k]; }
@@ -331,8 +331,8 @@ cudaError_t prepare_step(lbch_handle* h, int k)
         return k == 0 ? prepare_step_t<double, double, double, 32, 8>(h, k)
              : k == 1 ? prepare_step_t<double, double, double, 16, 8>(h, k)
              : k == 2 ? prepare_step_t<double, double, double, 32, 8, 512>(h, k)
-             : k == 3 ? prepare_step_t<double, double, double, 32, 16, 736>(h, k)
-                      : prepare_step_t<double, double, double, 32, 14, 672>(h, k);
+             : k == 3 ? prepare_step_t<double, double, double, 32, 16, 768>(h, k)
+                      : prepare_step_t<double, double, double, 32, 14, 704>(h, k);
     case LBCH_F32:
         return k == 0 ? prepare_step_t<float, float, float, 32, 16>(h, k)
              : k == 1 ? prepare_step_t<float, float, float, 32, 8>(h, k)
@@ -419,8 +419,8 @@ cudaError_t launch_step(lbch_handle* h, int parity)
         return k == 0 ? launch_step_t<double, double, double, 32, 8>(h, parity)
              : k == 1 ? launch_step_t<double, double, double, 16, 8>(h, parity)
              : k == 2 ? launch_step_t<double, double, double, 32, 8, 512>(h, parity)
-             : k == 3 ? launch_step_t<double, double, double, 32, 16, 736>(h, parity)
-                      : launch_step_t<double, double, double, 32, 14, 672>(h, parity);
+             : k == 3 ? launch_step_t<double, double, double, 32, 16, 768>(h, parity)
+                      : launch_step_t<double, double, double, 32, 14, 704>(h, parity);
     case LBCH_F32:
         return k == 0 ? launch_step_t<float, float, float, 32, 16>(h, parity)
              : k == 1 ? launch_step_t<float, float, float, 32, 8>(h, parity)

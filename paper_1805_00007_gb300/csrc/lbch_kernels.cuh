@@ -549,7 +549,11 @@ struct StepShape {
     static constexpr size_t OFF_P = a128(GBOX_BYTES), OFF_L = OFF_P + a128(PBOX_BYTES);
     static constexpr size_t OFF_T = OFF_L + a128(LBOX_BYTES);
     static constexpr size_t STAGE = OFF_T + a128(TAB_BYTES);
-    static constexpr size_t WORK1 = a128(sizeof(C) * (2 * NM));
+    // the column passes of the double path: five column values of phi on tile + 3 by tile + 2 rows (then four of mu and D)
+    static constexpr int AW = TX + 6, AN = AW * MH;
+    static constexpr bool COLS = sizeof(C) == 8;
+    static constexpr size_t OFF_COLS = a128(sizeof(C) * (2 * NM));
+    static constexpr size_t WORK1 = OFF_COLS + (COLS ? a128(sizeof(C) * (5 * AN)) : 0);
     static constexpr size_t WORK = WORK1 + (sizeof(S) == 2 ? a128(sizeof(C) * NG) : 0);  // + h*_0 (half path)
     static constexpr size_t BYTES = 2 * STAGE + WORK + 128 + 128;  // mbarriers, alignment slack
 };
@@ -694,6 +698,35 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         }
 
         // 2. mu (Eq. mu) and D = div(phi u) on tile + 2
+        // In double the stencils go through shared memory column first (lbch_kernels.cuh, per-node arithmetic): a pass for
+        // the column values, then one along the rows, for phi and again for mu and D.  Two more barriers, but no
+        // column value is formed three times, and it is the FP64 pipe that bounds these kernels (32 x 14
+        // tiles at 256^2: 19.7 -> 16.0 us per step, 500^2 74.3 -> 59.3, about three quarters of the pipe's rate).
+        // In float, where latency does, every thread forms what it needs from the nine neighbours.
+        C* s_z = s_mu + L::OFF_COLS / sizeof(C);
+        if constexpr (L::COLS) {
+            constexpr int AW = L::AW, AN = L::AN;
+            for_region<AW, MH, AW, NT>([&](int e, int r, int c) {
+                const P* q = pb + (r + 1) * BW + c + 1;
+                const C pS = cvt<C>(q[-BW]), ce = cvt<C>(q[0]), pN = cvt<C>(q[BW]);
+                C dl;
+                s_z[e] = node_z(pS, ce, pN, dl);
+                s_z[AN + e] = dl;
+                if (model >= 2) {
+                    C E, W;
+                    s_z[2 * AN + e] = node_flux(pS, ce, pN, sX1[c + 1], sX2[c + 1], sY1[r], op_mul(C(4), sY1[r + 1]), sY1[r + 2],
+                                                sY2[r], sY2[r + 2], E, W);
+                    s_z[3 * AN + e] = E;
+                    s_z[4 * AN + e] = W;
+                }
+            });
+            __syncthreads();
+            for_region<MW, L::MH, MW, NT>([&](int e, int r, int c) {
+                const int k = r * AW + c + 1;
+                s_mu[e] = node_mu(cvt<C>(pb[(r + 1) * BW + c + 2]), s_z[AN + k], s_z[k], s_z[k + 1], s_z[k - 1], K0);
+                if (model >= 2) s_D[e] = node_div(s_z[2 * AN + k], s_z[3 * AN + k + 1], s_z[4 * AN + k - 1]);
+            });
+        } else
         // (the compact order in every phase: the strided order of for_region measured no faster here, 4.56
         // against 4.55 us per step for 256^2 at tau_g = 0.8 in FP32, 4.30 against 4.23 with half storage)
         for_region<MW, L::MH, MW, NT>([&](int e, int r, int c) {
@@ -724,17 +757,43 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         }
         __syncthreads();
 
+        // the column values of mu and D (in the place of phi's)
+        constexpr int CN = MW * L::GH;
+        if constexpr (L::COLS) {
+            for_region<MW, L::GH, MW, NT>([&](int e, int r, int c) {
+                const C mS = s_mu[e], mN = s_mu[e + 2 * MW];
+                s_z[e] = node_w(mS, s_mu[e + MW], mN);
+                s_z[CN + e] = mN - mS;
+                if (model >= 2) {
+                    const C dS = s_D[e], dN = s_D[e + 2 * MW];
+                    s_z[2 * CN + e] = node_w(dS, s_D[e + MW], dN);
+                    s_z[3 * CN + e] = dN - dS;
+                }
+            });
+            __syncthreads();
+        }
+
         // 3. force, equilibrium, source and collision on tile + 1, written back into the box
         for_region<GW, L::GH, GW, NT>([&](int e, int r, int c) {
             int gy = y0 - 1 + r;
             if (walls && (gy < 0 || gy >= ny)) return;  // ghost rows: never pulled (bounce-back)
             int m = (r + 1) * MW + (c + 1);
             C gmx, gmy, gDx = C(0), gDy = C(0);
-            grad9(s_mu[m + 1], s_mu[m - 1], s_mu[m + MW], s_mu[m - MW], s_mu[m + MW + 1], s_mu[m + MW - 1],
-                  s_mu[m - MW + 1], s_mu[m - MW - 1], gmx, gmy);
-            if (model >= 2)
-                grad9(s_D[m + 1], s_D[m - 1], s_D[m + MW], s_D[m - MW], s_D[m + MW + 1], s_D[m + MW - 1],
-                      s_D[m - MW + 1], s_D[m - MW - 1], gDx, gDy);
+            if constexpr (L::COLS) {
+                const C* w = s_z + r * MW + c + 1;
+                gmx = w[1] - w[-1];
+                gmy = node_gy(w[CN - 1], w[CN], w[CN + 1]);
+                if (model >= 2) {
+                    gDx = w[2 * CN + 1] - w[2 * CN - 1];
+                    gDy = node_gy(w[3 * CN - 1], w[3 * CN], w[3 * CN + 1]);
+                }
+            } else {
+                grad9(s_mu[m + 1], s_mu[m - 1], s_mu[m + MW], s_mu[m - MW], s_mu[m + MW + 1], s_mu[m + MW - 1],
+                      s_mu[m - MW + 1], s_mu[m - MW - 1], gmx, gmy);
+                if (model >= 2)
+                    grad9(s_D[m + 1], s_D[m - 1], s_D[m + MW], s_D[m - MW], s_D[m + MW + 1], s_D[m + MW - 1],
+                          s_D[m - MW + 1], s_D[m - MW - 1], gDx, gDy);
+            }
             C ph = cvt<C>(pb[(r + 2) * BW + c + 3]);
             C mu = s_mu[m];
             const C ux = node_u(sX1[c + 3], sY1[r + 2]), uy = node_u(sX2[c + 3], sY2[r + 2]);  // box row r+2, col c+3
