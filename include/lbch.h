@@ -172,10 +172,11 @@ lbch_status lb_ch_halo_import(lbch_handle* h, int side, const void* src);
  * is enqueued (in CUDA graphs of 64 steps when possible) and the call returns.  When every instance has
  * tau_g = 1 (the paper's default), Eq. LB reduces to g* = g_eq + S/2 and the populations drop out of the
  * step: the library then reads and writes phi only (the stored populations are left unchanged and are
- * not part of the state), with the same results bit for bit.  Until lb_ch_tune chooses otherwise, a
- * handle whose instances are all periodic with tau_g = 1 (LBCH_F32 or LBCH_F64) and whose grid fits the
- * device in one wave of two-step tiles (up to about 68 K nodes) steps two steps per launch
- * with the two-step kernel; every other handle steps with the row sweep. */
+ * not part of the state), with the same results bit for bit.  Until lb_ch_tune chooses otherwise, the
+ * kernel is chosen by the size of the handle's grids: LBCH_F32 handles whose instances are all periodic with tau_g = 1
+ * and fit the device in two waves of two-step tiles (up to about 150 K nodes) step two steps per launch with the two-step
+ * kernel; the tile kernel steps LBCH_F64 handles of up to about 900 K nodes and, where some tau_g != 1, float ones of up
+ * to about 75 K; the row sweep steps every other handle, and those with a Model III instance. */
 lbch_status lb_ch_step(lbch_handle* h, long nsteps);
 
 /* Read an observable of instance inst into out (host, sized as lbch_obs states).  Synchronises the

@@ -1043,6 +1043,48 @@ cudaError_t adjoint_end_t(lbch_handle* h, C* dphi0)
     return cudaGetLastError();
 }
 
+// The kernel that steps a handle until lb_ch_tune measures: by the number of its tiles against the SMs, from the times of
+// every form and shape on grids of 48^2 to 4096^2 (one GB300, us per step).
+void choose_default(lbch_handle* h, int sms)
+{
+    if (h->coupled) return;
+    const bool tau1 = h->tau1;
+    // the row sweep: on grids so small that sixteen warps per SM would get two rows each or fewer, strips for half as many
+    // warps (eight in double: a quarter) step faster -- 256^2 in float 4.7 against 5.3, double 36 against 54
+    const lbch_handle::SweepCut& cut = h->sw[0][sweep_gen(h)];
+    h->shape = h->prec == LBCH_F64 ? (cut.rows_per <= 8 && !h->model3 ? 2 : 0) : (cut.rows_per <= 2 ? 1 : 0);
+    if (h->model3) return;
+    auto tiles = [&](int k) { return h->ps[k].total_tiles; };
+    if (h->prec == LBCH_F64) {
+        // The tile kernel while its waves are few, where strips would be short (500^2: 59 against 69); the row sweep on
+        // grids of a dozen waves (1024^2 at tau_g = 1: 223 against 229; 724^2: 121 against 115).  Small grids take the
+        // smallest tiles that leave no SM two of them (100^2: 7.8 against 16.0 with 32 x 14), others the shape of
+        // the least waves times the time of one (32 x 16: 16.7 at tau_g = 1, 32 x 14: 14.9).
+        if (tiles(3) > 12 * sms) return;
+        h->force_tile = true;
+        auto waves = [&](int k) { return (tiles(k) + sms - 1) / sms; };
+        h->shape = tiles(1) <= sms ? 1 : tiles(2) <= sms ? 2 : waves(4) * 149 <= waves(3) * 167 ? 4 : 3;
+        return;
+    }
+    if (h->prec == LBCH_F16S && tau1) return;  // the tile kernel would round the populations to half
+    if (!tau1) {
+        // with the populations: small tiles on small grids (100^2: 3.0 against the sweep's 3.6; 160^2: 3.5), one wave of
+        // 32 x 16 (256^2: 4.6 against 5.8), then the row sweep (360^2: 7.1 against 7.4)
+        if (2 * tiles(2) <= 3 * sms) { h->force_tile = true; h->shape = 2; }
+        else if (tiles(3) <= sms) { h->force_tile = true; h->shape = 3; }
+        return;
+    }
+    // tau_g = 1 in float: the two-step kernel on periodic grids up to two waves of its tiles -- 32 x 8 (100^2: 1.9 per
+    // step against the row sweep's 4.0), one of 32 x 14 (256^2: 2.55 against 4.7), two of 32 x 16 (360^2: 4.7 against
+    // 5.5) --, otherwise the row sweep (512^2: 6.2 against 8.9).  The odd last step of a call, and taped steps, take
+    // the one-step kernel that is faster there: 16 x 8 tiles up to three per SM (100^2: 2.7 against 4.0).
+    if (!pair_ok(h)) return;
+    auto pairs = [&](int k) { return h->pr[k].total_tiles; };
+    h->pshape = pairs(3) <= sms ? 3 : pairs(1) <= sms ? 1 : 2;
+    h->pair = pairs(h->pshape) <= 2 * sms;
+    if (h->pair && tiles(2) <= 3 * sms) { h->force_tile = true; h->shape = 2; }
+}
+
 // lb_ch_init and lb_ch_init_slab.  With a slab, params is the one instance of the slab (the global problem
 // with ny = slab->ny), gparams the global problem (for the velocity tables), and phi0 holds slab->ny + 2 GR
 // rows: the slab's rows with GR rows of each neighbour (global rows y0 - GR .. y0 + ny + GR - 1, wrapped).
@@ -1158,6 +1200,8 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
         CKI(cudaMemcpyAsync(h->ps[sk].d_tile_begin, tile_begin[sk].data(), sizeof(int) * (n_inst + 1),
                             cudaMemcpyHostToDevice, h->stream));
     }
+    int sms = 0;
+    CKI(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     if (!coupled) {
         for (int gen = h->tau1 ? 0 : 1; gen < 2; gen++) {  // (with tau_g = 1 the populations are kept for tests only)
             SweepFit fit;
@@ -1311,14 +1355,7 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     }
     CKI(cudaStreamSynchronize(h->stream));  // the pinned staging buffer and the tables are reused after this
 #undef CKI
-    // Kernel before any tuning: the two-step kernel where it applies and its tiles fit the device in one
-    // wave (a step of such a grid is bound by latency, and one launch per two steps halves the launches);
-    // otherwise the row sweep.  lb_ch_tune measures instead.
-    const int k2 = prec == LBCH_F64 ? 3 : 1;  // 32 x 14 tiles in either precision
-    if (pair_ok(h) && h->pr[k2].d_tile_begin && h->pr[k2].grid == h->pr[k2].total_tiles) {
-        h->pair = true;
-        h->pshape = k2;
-    }
+    choose_default(h, sms);
     *out = h;
     return LBCH_OK;
 }
