@@ -14,8 +14,9 @@
 // in double for every storage precision (at tau = 1 all nine lambda_q are equal and dL/du is formed from
 // differences of neighbouring lambda, which float storage would round away); the tape keeps the
 // forward phi in the precision of the forward path, so the gradient is that of the path actually run.
-// Four one-thread-per-node kernels per adjoint step (forward mu; local adjoints; mu_bar and D_bar; phi_bar
-// and the new lambda), and one deterministic sum of dL/ds at the end of the sweep.
+// Two kernels per adjoint step on tiles of 32 x 8 nodes (local_kernel: forward mu and the local adjoints of collision,
+// g_eq, S and F1; transpose_kernel: mu_bar and D_bar on tile + 1, phi_bar and the new lambda), and one deterministic sum of
+// dL/ds at the end of the sweep.
 //
 // CF: the type the forward quantities are formed in (mu, its gradient, the velocity, rho and the force's
 // coefficient, f''(phi)) -- float for a float tape, as the float forward step formed them, double for a double
@@ -37,6 +38,8 @@ struct AdjArgs {
     int pitch;                 // of the velocity tables' X part
     int ylen;                  // length of each Y table
     long long n;               // forward step index of this adjoint step
+    // constants of the adjoint step, formed once on the host: src/12, eta/tau, src/144, -K src/144
+    double s12, ieta, s144, sK144;
 };
 
 __device__ __forceinline__ int wp(int i, int n) { return i >= n ? i - n : (i < 0 ? i + n : i); }
@@ -90,21 +93,13 @@ __device__ __forceinline__ void geq_contract(const C* l, C phi, C ux, C uy, C et
     by = phi * (C(3) * m1y + C(9) * vy - C(3) * uy * m0);
 }
 
-// The isotropic stencils on the periodic lattice, grouped by axis and diagonal neighbours:
-// (G v)(x) = sum_k w_k c_k v(x + c_k)/c_s^2 and (L v)(x) = sum_k 2 w_k (v(x + c_k) - v(x))/c_s^2.  Their
-// transposes follow by substituting c_k -> -c_k: G^T = -G and L^T = L.
+// The isotropic Laplacian on the periodic lattice, grouped by axis and diagonal neighbours:
+// (L v)(x) = sum_k 2 w_k (v(x + c_k) - v(x))/c_s^2.  Its transpose follows by substituting c_k -> -c_k: L^T = L (and
+// G^T = -G for the gradient).
 template <typename C, typename V>
 __device__ __forceinline__ C at_nb(const V* v, int nx, int ny, int x, int y, int dx, int dy)
 {
     return (C)v[(long long)wp(y + dy, ny) * nx + wp(x + dx, nx)];
-}
-template <typename C, typename V>
-__device__ __forceinline__ C grad_c(const V* v, int nx, int ny, int x, int y, int comp)
-{
-    auto at = [&](int dx, int dy) { return at_nb<C>(v, nx, ny, x, y, dx, dy); };
-    if (comp == 0)
-        return C(1) / C(3) * (at(1, 0) - at(-1, 0)) + C(1) / C(12) * ((at(1, 1) - at(-1, 1)) + (at(1, -1) - at(-1, -1)));
-    return C(1) / C(3) * (at(0, 1) - at(0, -1)) + C(1) / C(12) * ((at(1, 1) + at(-1, 1)) - (at(1, -1) + at(-1, -1)));
 }
 template <typename C, typename V>
 __device__ __forceinline__ C lap_c(const V* v, int nx, int ny, int x, int y)
@@ -115,12 +110,6 @@ __device__ __forceinline__ C lap_c(const V* v, int nx, int ny, int x, int y)
     const C dg = (at(1, 1) + at(-1, 1)) + (at(1, -1) + at(-1, -1));
     return C(2) / C(3) * (ax - C(4) * c) + C(1) / C(6) * (dg - C(4) * c);
 }
-// (G^T v)(x), component comp
-template <typename C>
-__device__ __forceinline__ C gradT(const C* v, int nx, int ny, int x, int y, int comp)
-{
-    return -grad_c<C>(v, nx, ny, x, y, comp);
-}
 // (L^T v)(x)
 template <typename C>
 __device__ __forceinline__ C lapT(const C* v, int nx, int ny, int x, int y)
@@ -128,114 +117,254 @@ __device__ __forceinline__ C lapT(const C* v, int nx, int ny, int x, int y)
     return lap_c<C>(v, nx, ny, x, y);
 }
 
-// forward mu = f'(phi) - kappa lap phi at step n (phi from the tape, of type TP), in the forward type CF
-template <typename CF, typename TP>
-__global__ void fwd_mu_kernel(const InstDev* inst, AdjArgs a, const TP* phi, CF* mu)
+// ---- one adjoint step
+//
+// Everything that carries lambda is bound by the FP64 pipe, so the two kernels are built to take few operations: about 90
+// per node, conversions of the forward quantities included, where four one-thread-per-node kernels took about 130 (us per
+// step with a float tape: 512^2 84 -> 56, 1024^2 281 -> 189, 100^2 25 -> 19; the pipe is 83 % busy).
+//   - The stencils go through shared memory column first (lbch_kernels.cuh): a pass for the column values, then one
+//     along the rows.
+//   - The moments of the gathered lambda' are stencils too.  With ONE they are, times 36: M0 = w(E) + 4 w + w(W),
+//     M1 = (w(E) - w(W), d(E) + 4 d + d(W)), M2xx = w(E) + w(W), M2yy = v(E) + 4 v + v(W), M2xy = d(E) - d(W) with the column
+//     values v = l(N) + l(S), w = 4 l + v, d = l(N) - l(S).
+//   - With B = M1 + (3 M2 - M0) u, the contractions of lambda' with d g_eq (geq_contract) are d/du: phi B/12 and
+//     d/dphi: l_0 + u.(B + M1)/24.  u.B is all that dL/ds needs of the former, so that one value is handed on.
+//   - S is linear in F: F_bar = src M1/12, so grad_mu_bar = -coef F_bar and D_bar = K G^T F_bar come from M1, which
+//     the first kernel hands to the second.
+// What is handed on: M1 (two values), the local phi_bar, the local mu_bar and u.B/tau.
+// Tiles of 32 x 8, one node per thread: four to six blocks per SM keep the pipe fed across each other's barriers, and
+// 1024 of them at 512^2 spread evenly (32 x 16 recompute less of the halo but took 66 us per step there, 32 x 4 65).
+constexpr int TX = 32, TY = 8, NT = 256;
+// transpose_kernel's shared memory: the vectors on tile + 2, later mu_bar and D_bar on tile + 1 with their column values
+constexpr int N_VEC = 4 * (TX + 4) * (TY + 4), N_BAR = 2 * (TX + 2) * (TY + 2) + 4 * (TX + 2) * TY;
+constexpr int N_FIRST = N_VEC > N_BAR ? N_VEC : N_BAR;
+constexpr size_t TRANSPOSE_SMEM = 8 * (N_FIRST + 6 * (TX + 4) * (TY + 2));
+
+__device__ __forceinline__ int wrap_any(int v, int n)
 {
-    const InstDev& I = inst[0];
-    const Consts<CF>& K0 = consts<CF>(I);
-    long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (long long)a.nx * a.ny) return;
-    int y = (int)k / a.nx, x = (int)k - y * a.nx;  // fewer than 2^31 nodes (lb_ch_adjoint_begin checks)
-    mu[k] = dfdphi((CF)phi[k], K0.beta, K0.phiA, K0.phiB) - K0.kappa * lap_c<CF>(phi, a.nx, a.ny, x, y);
+    if (v < 0 || v >= n) {
+        v %= n;
+        if (v < 0) v += n;
+    }
+    return v;
 }
 
-// local adjoints of collision, g_eq, S and F1 (lambda itself is written by transpose2_kernel)
-template <typename C, typename CF, typename TP, bool ONE>
-__global__ void local_kernel(const InstDev* inst, const CF* tabs, AdjArgs a, CF T, const TP* phi, const CF* mu,
-                             const C* lam_next, C* lam, C* gmb, C* Fb, C* phib, C* mub, C* ub)
+// f(e, i, j) for the nodes (i, j) of a W x H region, e = j W + i
+template <int W, int H, typename F> __device__ __forceinline__ void region(F&& f)
 {
+    for (int e = threadIdx.x; e < W * H; e += NT) {
+        const int j = e / W;
+        f(e, e - j * W, j);
+    }
+}
+
+template <typename C, typename CF, typename TP, bool ONE>
+__global__ void __launch_bounds__(NT, ONE ? 4 : 3) local_kernel(const InstDev* inst, const CF* tabs, AdjArgs a, CF T, const TP* phi,
+                                                      const C* lam_next, C* M1, C* phib, C* mub, C* uB)
+{
+    constexpr int PW = TX + 4, PH = TY + 4;  // phi on tile + 2
+    constexpr int ZW = TX + 4, ZH = TY + 2;  // its column values
+    constexpr int MW = TX + 2, MH = TY + 2;  // mu (and lambda) on tile + 1
+    constexpr int GW = TX + 2, GH = TY;      // the column values of mu (and lambda)
+    __shared__ CF s_p[PW * PH], s_z[ZW * ZH], s_dl[ZW * ZH], s_m[MW * MH], s_wm[GW * GH], s_dm[GW * GH];
+    __shared__ C s_l[ONE ? MW * MH : 1], s_v[ONE ? GW * GH : 1], s_w[ONE ? GW * GH : 1], s_d[ONE ? GW * GH : 1];
     const InstDev& I = inst[0];
     const Consts<C>& K0 = consts<C>(I);
     const Consts<CF>& KF = consts<CF>(I);
-    const long long N = (long long)a.nx * a.ny;
-    long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= N) return;
-    int y = (int)k / a.nx, x = (int)k - y * a.nx;  // fewer than 2^31 nodes (lb_ch_adjoint_begin checks)
-    // the forward quantities at the node, in CF
-    const CF phf = (CF)phi[k];
-    CF uxf, uyf;
-    vel_at(I, tabs, a, x, y, T, uxf, uyf);
-    const CF gxf = grad_c<CF>(mu, a.nx, a.ny, x, y, 0), gyf = grad_c<CF>(mu, a.nx, a.ny, x, y, 1);  // grad mu
-    const CF rhof = KF.a * phf + KF.b, rf = rcp<CF>(rhof);
-    const CF coeff = phf * phf * rf;                                    // F1 = -coef grad mu
-    const CF dcoeff = phf * (KF.a * phf + CF(2) * KF.b) * (rf * rf);   // d coef / d phi
-    const C ph = (C)phf, ux = (C)uxf, uy = (C)uyf, gx = (C)gxf, gy = (C)gyf, coef = (C)coeff, dcoef = (C)dcoeff;
-    C pb[9];
+    const int nx = a.nx, ny = a.ny;
+    const long long N = (long long)nx * ny;
+    const int tiles_x = (nx + TX - 1) / TX;
+    const int x0 = ((int)blockIdx.x % tiles_x) * TX, y0 = ((int)blockIdx.x / tiles_x) * TY;
+    region<PW, PH>([&](int e, int i, int j) {
+        s_p[e] = (CF)phi[(long long)wrap_any(y0 - 2 + j, ny) * nx + wrap_any(x0 - 2 + i, nx)];
+    });
+    if constexpr (ONE)
+        region<MW, MH>([&](int e, int i, int j) {
+            s_l[e] = lam_next[(long long)wrap_any(y0 - 1 + j, ny) * nx + wrap_any(x0 - 1 + i, nx)];
+        });
+    __syncthreads();
+    region<ZW, ZH>([&](int e, int i, int j) {
+        CF dl;
+        s_z[e] = node_z(s_p[e], s_p[e + PW], s_p[e + 2 * PW], dl);
+        s_dl[e] = dl;
+    });
+    if constexpr (ONE)
+        region<GW, GH>([&](int e, int i, int j) {
+            const C S = s_l[e], Nn = s_l[e + 2 * MW];
+            const C v = Nn + S;
+            s_v[e] = v;
+            s_w[e] = fma(C(4), s_l[e + MW], v);
+            s_d[e] = Nn - S;
+        });
+    __syncthreads();
+    region<MW, MH>([&](int e, int i, int j) {
+        const int k = j * ZW + i + 1;
+        s_m[e] = node_mu(s_p[k + PW], s_dl[k], s_z[k], s_z[k + 1], s_z[k - 1], KF);
+    });
+    __syncthreads();
+    region<GW, GH>([&](int e, int i, int j) {
+        const CF S = s_m[e], Nn = s_m[e + 2 * MW];
+        s_wm[e] = node_w(S, s_m[e + MW], Nn);
+        s_dm[e] = Nn - S;
+    });
+    __syncthreads();
+    region<TX, TY>([&](int e, int i, int j) {
+        const int x = x0 + i, y = y0 + j;
+        if (x >= nx || y >= ny) return;
+        const long long k = (long long)y * nx + x;
+        const int c = j * GW + i + 1;  // the node among the column values
+        // the forward quantities at the node, in CF
+        const CF phf = s_p[(j + 2) * PW + i + 2];
+        CF uxf, uyf;
+        vel_at(I, tabs, a, x, y, T, uxf, uyf);
+        const CF gxf = op_mul(CF(1) / CF(12), s_wm[c + 1] - s_wm[c - 1]);  // grad mu
+        const CF gyf = op_mul(CF(1) / CF(12), node_gy(s_dm[c - 1], s_dm[c], s_dm[c + 1]));
+        const CF rhof = KF.a * phf + KF.b, rf = rcp<CF>(rhof);
+        const CF dcoeff = phf * (KF.a * phf + CF(2) * KF.b) * (rf * rf);  // d coef / d phi, F1 = -coef grad mu
+        const C ux = (C)uxf, uy = (C)uyf, gx = (C)gxf, gy = (C)gyf, dcoef = (C)dcoeff;
+        // 36 times the moments of lambda'_q = lambda_q(x + c_q) (reverse streaming)
+        C l0, M0, M1x, M1y, Mxx, Myy, Mxy;
+        if constexpr (ONE) {
+            l0 = s_l[(j + 1) * MW + i + 1];
+            const C dE = s_d[c + 1], d = s_d[c], dW = s_d[c - 1], wE = s_w[c + 1], wW = s_w[c - 1];
+            Mxx = wE + wW;
+            M0 = fma(C(4), s_w[c], Mxx);
+            M1x = wE - wW;
+            M1y = fma(C(4), d, dE + dW);
+            Myy = fma(C(4), s_v[c], s_v[c + 1] + s_v[c - 1]);
+            Mxy = dE - dW;
+        } else {
+            C l[9];
 #pragma unroll
-    for (int q = 0; q < 9; q++) {
-        // reverse streaming: post_q(x) was sent to x + c_q
-        pb[q] = lam_next[(ONE ? 0 : q * N) + (long long)wp(y + cy(q), a.ny) * a.nx + wp(x + cx(q), a.nx)];
-    }
-    // post_q takes g_eq_q / tau and (1 - 1/(2 tau)) S_q, S_q = w_q c_q . F / c_s^2
-    C pl, ml, bx, by, m1x, m1y;
-    geq_contract(pb, ph, ux, uy, K0.eta, pl, ml, bx, by, m1x, m1y);
-    pl *= K0.itau;
-    ml *= K0.itau;
-    bx *= K0.itau;
-    by *= K0.itau;
-    const C fbx = C(3) * K0.src * m1x, fby = C(3) * K0.src * m1y;
-    gmb[k] = -coef * fbx;
-    gmb[N + k] = -coef * fby;
-    Fb[k] = fbx;
-    Fb[N + k] = fby;
-    phib[k] = pl - dcoef * (fbx * gx + fby * gy);
-    mub[k] = ml;
-    ub[k] = bx;
-    ub[N + k] = by;
+            for (int q = 0; q < 9; q++)
+                l[q] = lam_next[q * N + (long long)wp(y + cy(q), ny) * nx + wp(x + cx(q), nx)];
+            // opposite pairs (1, 3) c = (1, 0); (2, 4) c = (0, 1); (5, 7) c = (1, 1); (6, 8) c = (-1, 1)
+            const C E1 = l[1] + l[3], O1 = l[1] - l[3], E2 = l[2] + l[4], O2 = l[2] - l[4];
+            const C E5 = l[5] + l[7], O5 = l[5] - l[7], E6 = l[6] + l[8], O6 = l[6] - l[8];
+            const C s56 = E5 + E6;
+            l0 = l[0];
+            Mxx = fma(C(4), E1, s56);
+            Myy = fma(C(4), E2, s56);
+            Mxy = E5 - E6;
+            M0 = fma(C(16), l0, fma(C(4), E2, Mxx));
+            M1x = fma(C(4), O1, O5 - O6);
+            M1y = fma(C(4), O2, O5 + O6);
+        }
+        const C r = C(3) * Mxy;
+        const C Bx = fma(ux, fma(C(3), Mxx, -M0), fma(uy, r, M1x));
+        const C By = fma(uy, fma(C(3), Myy, -M0), fma(ux, r, M1y));
+        const C ub = fma(ux, Bx, uy * By), um = fma(ux, M1x, uy * M1y);
+        const C pl = fma(C(1) / C(24), ub + um, l0);            // sum_q l_q d g_eq_q/d phi
+        const C ml = fma(C(1) / C(36), M0, -l0);                // (1/eta) sum_q l_q d g_eq_q/d mu
+        M1[k] = M1x;
+        M1[N + k] = M1y;
+        phib[k] = fma(K0.itau, pl, -(C(a.s12) * dcoef) * fma(M1x, gx, M1y * gy));
+        mub[k] = C(a.ieta) * ml;
+        uB[k] = K0.itau * ub;
+    });
 }
 
-// mu_bar += G^T grad_mu_bar;  D_bar = 3 c_s^2 K G^T F_bar
-template <typename C>
-__global__ void transpose1_kernel(const InstDev* inst, AdjArgs a, const C* gmb, const C* Fb, C* mub, C* Db)
-{
-    const InstDev& I = inst[0];
-    const Consts<C>& K0 = consts<C>(I);
-    const long long N = (long long)a.nx * a.ny;
-    long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= N) return;
-    int y = (int)k / a.nx, x = (int)k - y * a.nx;  // fewer than 2^31 nodes (lb_ch_adjoint_begin checks)
-    mub[k] += gradT(gmb, a.nx, a.ny, x, y, 0) + gradT(gmb + N, a.nx, a.ny, x, y, 1);
-    Db[k] = (a.model == 2) ? K0.K * (gradT(Fb, a.nx, a.ny, x, y, 0) + gradT(Fb + N, a.nx, a.ny, x, y, 1)) : C(0);
-}
-
+// mu_bar = local + G^T grad_mu_bar;  D_bar = 3 c_s^2 K G^T F_bar;
 // phi_bar = local + f''(phi) mu_bar - kappa L^T mu_bar + u . G^T D_bar;
-// lambda_q(x) = (1 - 1/tau) lambda_next_q(x + c_q) + phi_bar(x); dL/ds per node
+// lambda_q(x) = (1 - 1/tau) lambda_next_q(x + c_q) + phi_bar(x); dL/ds per node.  (G^T = -G, L^T = L.)
 template <typename C, typename CF, typename TP, bool ONE>
-__global__ void transpose2_kernel(const InstDev* inst, const CF* tabs, AdjArgs a, CF T, const TP* phi,
-                                  const C* phib, const C* mub, const C* Db, const C* ub, const C* lam_next, C* lam,
-                                  double* ds)
+__global__ void __launch_bounds__(NT, ONE ? 6 : 3) transpose_kernel(const InstDev* inst, const CF* tabs, AdjArgs a, CF T,
+                                                          const TP* phi, const C* M1, const C* phib, const C* mub,
+                                                          const C* uB, const C* lam_next, C* lam, double* ds)
 {
+    constexpr int VW = TX + 4, VH = TY + 4;  // M1 and coef M1 on tile + 2
+    constexpr int ZW = TX + 4, ZH = TY + 2;  // the column values of their divergences
+    constexpr int MW = TX + 2, MH = TY + 2;  // mu_bar, D_bar on tile + 1
+    constexpr int GW = TX + 2, GH = TY;      // their column values
+    constexpr int NV = VW * VH, NZ = ZW * ZH, NM = MW * MH, NG = GW * GH;
+    // the vectors, later (their place taken over) mu_bar, D_bar and their column values; the shares of the divergences
+    static_assert(4 * NV <= N_FIRST && 2 * NM + 4 * NG <= N_FIRST, "the first part holds either");
+    extern __shared__ __align__(16) unsigned char smem_adj[];
+    C *s_v = reinterpret_cast<C*>(smem_adj), *s_c = s_v + N_FIRST;
     const InstDev& I = inst[0];
     const Consts<C>& K0 = consts<C>(I);
     const Consts<CF>& KF = consts<CF>(I);
-    const long long N = (long long)a.nx * a.ny;
-    long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= N) return;
-    int y = (int)k / a.nx, x = (int)k - y * a.nx;  // fewer than 2^31 nodes (lb_ch_adjoint_begin checks)
-    // the forward quantities at the node, in CF
-    const CF phf = (CF)phi[k];
-    CF uxf, uyf;
-    vel_at(I, tabs, a, x, y, T, uxf, uyf);
-    const C ph = (C)phf, ux = (C)uxf, uy = (C)uyf;
-    const C f2 = (C)d2f(phf, KF.beta, KF.phiA, KF.phiB);
-    C pb = phib[k] + f2 * mub[k] - K0.kappa * lapT(mub, a.nx, a.ny, x, y);
-    C bx = ub[k], by = ub[N + k];
-    if (a.model == 2) {
-        C jbx = gradT(Db, a.nx, a.ny, x, y, 0), jby = gradT(Db, a.nx, a.ny, x, y, 1);
-        pb += ux * jbx + uy * jby;
-        bx += ph * jbx;
-        by += ph * jby;
-    }
-    // u = s u_ref: du/ds = u.  Accumulated per node over the adjoint steps and summed once at the end.
-    ds[k] += (double)bx * (double)ux + (double)by * (double)uy;
-    if constexpr (ONE) {
-        lam[k] = pb;  // (1 - 1/tau) = 0: the reverse streaming and collision leave phi_bar alone
-    } else {
+    const int nx = a.nx, ny = a.ny;
+    const long long N = (long long)nx * ny;
+    const int tiles_x = (nx + TX - 1) / TX;
+    const int x0 = ((int)blockIdx.x % tiles_x) * TX, y0 = ((int)blockIdx.x / tiles_x) * TY;
+    const bool model2 = a.model == 2;
+    region<VW, VH>([&](int e, int i, int j) {
+        const long long k = (long long)wrap_any(y0 - 2 + j, ny) * nx + wrap_any(x0 - 2 + i, nx);
+        const CF phf = (CF)phi[k];
+        const C coef = (C)(phf * phf * rcp<CF>(KF.a * phf + KF.b));  // F1 = -coef grad mu
+        const C mx = M1[k], my = M1[N + k];
+        s_v[e] = coef * mx;
+        s_v[NV + e] = coef * my;
+        s_v[2 * NV + e] = mx;
+        s_v[3 * NV + e] = my;
+    });
+    __syncthreads();
+    // the share of a column in the divergence (times 12) of the node to its west, to its east and of its own node (times 4)
+    auto col = [&](const C* v, int e, C* o) {
+        const C t = fma(C(4), v[e + VW], v[e + 2 * VW] + v[e]), d = v[NV + e + 2 * VW] - v[NV + e];
+        o[e] = t + d;
+        o[NZ + e] = d - t;
+        o[2 * NZ + e] = d;
+    };
+    region<ZW, ZH>([&](int e, int i, int j) {
+        col(s_v, e, s_c);
+        if (model2) col(s_v + 2 * NV, e, s_c + 3 * NZ);
+    });
+    __syncthreads();
+    C *s_mu = s_v, *s_D = s_v + NM, *s_z = s_v + 2 * NM;  // the vectors are read no more
+    const C cm = C(a.s144), cD = C(a.sK144);
+    region<MW, MH>([&](int e, int i, int j) {
+        const int k = j * ZW + i + 1;
+        const long long g = (long long)wrap_any(y0 - 1 + j, ny) * nx + wrap_any(x0 - 1 + i, nx);
+        // grad_mu_bar = -coef src M1/12, and G^T is minus a twelfth of the sum of the shares
+        s_mu[e] = fma(cm, fma(C(4), s_c[2 * NZ + k], s_c[k + 1] + s_c[NZ + k - 1]), mub[g]);
+        if (model2) s_D[e] = cD * fma(C(4), s_c[5 * NZ + k], s_c[3 * NZ + k + 1] + s_c[4 * NZ + k - 1]);
+    });
+    __syncthreads();
+    region<GW, GH>([&](int e, int i, int j) {
+        const C S = s_mu[e], c = s_mu[e + MW], Nn = s_mu[e + 2 * MW];
+        C dl;
+        s_z[e] = node_z(S, c, Nn, dl);
+        s_z[NG + e] = dl;
+        if (model2) {
+            const C dS = s_D[e], dN = s_D[e + 2 * MW];
+            s_z[2 * NG + e] = node_w(dS, s_D[e + MW], dN);
+            s_z[3 * NG + e] = dN - dS;
+        }
+    });
+    __syncthreads();
+    region<TX, TY>([&](int e, int i, int j) {
+        const int x = x0 + i, y = y0 + j;
+        if (x >= nx || y >= ny) return;
+        const long long k = (long long)y * nx + x;
+        const int c = j * GW + i + 1;
+        // the forward quantities at the node, in CF
+        const CF phf = (CF)phi[k];
+        CF uxf, uyf;
+        vel_at(I, tabs, a, x, y, T, uxf, uyf);
+        const C ph = (C)phf, ux = (C)uxf, uy = (C)uyf;
+        const C f2 = (C)d2f(phf, KF.beta, KF.phiA, KF.phiB);
+        const C z = s_z[c], lap = s_z[NG + c] + fma(C(-2), z, s_z[c + 1] + s_z[c - 1]);
+        C pb = fma(-K0.kappa, lap, fma(f2, s_mu[(j + 1) * MW + i + 1], phib[k]));
+        C ub = uB[k];  // 12 u . (adjoint of phi u), to which 12 u . G^T D_bar adds
+        if (model2) {
+            const C* w = s_z + 2 * NG + c;
+            const C* d = s_z + 3 * NG + c;
+            const C uj = fma(ux, w[-1] - w[1], -(uy * fma(C(4), d[0], d[1] + d[-1])));
+            pb = fma(C(1) / C(12), uj, pb);
+            ub += uj;
+        }
+        // u = s u_ref: du/ds = u.  Accumulated per node over the adjoint steps and summed once at the end.
+        ds[k] = fma(C(1) / C(12), ph * ub, ds[k]);
+        if constexpr (ONE) {
+            lam[k] = pb;  // (1 - 1/tau) = 0: the reverse streaming and collision leave phi_bar alone
+        } else {
 #pragma unroll
-        for (int q = 0; q < 9; q++)  // reverse streaming and collision, plus phi = sum_q g_q
-            lam[q * N + k] = K0.omt * lam_next[q * N + (long long)wp(y + cy(q), a.ny) * a.nx + wp(x + cx(q), a.nx)] + pb;
-    }
+            for (int q = 0; q < 9; q++)  // reverse streaming and collision, plus phi = sum_q g_q
+                lam[q * N + k] = K0.omt * lam_next[q * N + (long long)wp(y + cy(q), ny) * nx + wp(x + cx(q), nx)] + pb;
+        }
+    });
 }
 
 // adjoint of the initial equilibria: dL/dphi0 (two kernels: local, then the mu transpose)

@@ -937,7 +937,7 @@ lbch_status halo_copy(lbch_handle* h, void* buf, int phi_row, int g_row, bool ou
 
 struct AdjView {  // pointers into the adjoint workspace
     void* lam[2];
-    void *mu, *gmb, *Fb, *phib, *mub, *Db, *ub;
+    void *M1, *phib, *mub, *uB;  // what local_kernel hands to transpose_kernel
     double* ds;
     double* dLds;
 };
@@ -953,13 +953,10 @@ AdjView adj_view(lbch_handle* h)
     auto take = [&](size_t n) { void* r = p; p += (n * e + 255) / 256 * 256; return r; };
     v.lam[0] = take(adj_planes(h) * N);
     v.lam[1] = take(adj_planes(h) * N);
-    v.mu = take(N);
-    v.gmb = take(2 * N);
-    v.Fb = take(2 * N);
+    v.M1 = take(2 * N);
     v.phib = take(N);
     v.mub = take(N);
-    v.Db = take(N);
-    v.ub = take(2 * N);
+    v.uB = take(N);
     v.ds = reinterpret_cast<double*>(p);
     p += (N * 8 + 255) / 256 * 256;
     v.dLds = reinterpret_cast<double*>(p);
@@ -970,7 +967,7 @@ size_t adj_bytes(const lbch_handle* h)
 {
     const size_t N = (size_t)h->inst[0].nx * h->inst[0].ny, e = h->adj_elem;
     auto r = [](size_t b) { return (b + 255) / 256 * 256; };
-    return 2 * r(adj_planes(h) * N * e) + r(N * e) + 2 * r(2 * N * e) + 3 * r(N * e) + r(2 * N * e) + r(N * 8) + 256;
+    return 2 * r(adj_planes(h) * N * e) + r(2 * N * e) + 3 * r(N * e) + r(N * 8) + 256;
 }
 
 adj::AdjArgs adj_args(const lbch_handle* h, long long n)
@@ -982,6 +979,11 @@ adj::AdjArgs adj_args(const lbch_handle* h, long long n)
     a.pitch = h->pitch;
     a.ylen = h->inst[0].ylen;
     a.n = n;
+    const Consts<double>& c = h->inst[0].cd;
+    a.s12 = c.src / 12.0;
+    a.ieta = c.itau * c.eta;
+    a.s144 = c.src / 144.0;
+    a.sK144 = -c.K * c.src / 144.0;
     return a;
 }
 
@@ -1007,22 +1009,20 @@ cudaError_t adjoint_step_t(lbch_handle* h, const TP* phi_n, long long n)
     using CF = TP;
     AdjView v = adj_view(h);
     adj::AdjArgs a = adj_args(h, n);
-    const long long N = (long long)a.nx * a.ny;
-    const int nb = (int)((N + 255) / 256);
+    const int nb = ((a.nx + adj::TX - 1) / adj::TX) * ((a.ny + adj::TY - 1) / adj::TY);
     const CF T = (CF)vel_t(h->inst[0].vel, h->inst[0].Tper, n);
     const CF* tabs = tables<CF>(h);
     const C* lam_next = static_cast<const C*>(v.lam[h->adj_par]);
     C* lam = static_cast<C*>(v.lam[h->adj_par ^ 1]);
-    adj::fwd_mu_kernel<CF, TP><<<nb, 256, 0, h->stream>>>(h->d_inst, a, phi_n, (CF*)v.mu);
     const bool one = adj_planes(h) == 1;
-    (one ? adj::local_kernel<C, CF, TP, true> : adj::local_kernel<C, CF, TP, false>)<<<nb, 256, 0, h->stream>>>(
-        h->d_inst, tabs, a, T, phi_n, (const CF*)v.mu, lam_next, lam, (C*)v.gmb, (C*)v.Fb, (C*)v.phib, (C*)v.mub,
-        (C*)v.ub);
-    adj::transpose1_kernel<C><<<nb, 256, 0, h->stream>>>(h->d_inst, a, (const C*)v.gmb, (const C*)v.Fb, (C*)v.mub,
-                                                         (C*)v.Db);
-    (one ? adj::transpose2_kernel<C, CF, TP, true> : adj::transpose2_kernel<C, CF, TP, false>)<<<nb, 256, 0, h->stream>>>(
-        h->d_inst, tabs, a, T, phi_n, (const C*)v.phib, (const C*)v.mub, (const C*)v.Db, (const C*)v.ub, lam_next,
-        lam, v.ds);
+    (one ? adj::local_kernel<C, CF, TP, true> : adj::local_kernel<C, CF, TP, false>)<<<nb, adj::NT, 0, h->stream>>>(
+        h->d_inst, tabs, a, T, phi_n, lam_next, (C*)v.M1, (C*)v.phib, (C*)v.mub, (C*)v.uB);
+    const auto transpose = one ? adj::transpose_kernel<C, CF, TP, true> : adj::transpose_kernel<C, CF, TP, false>;
+    cudaError_t e = lbch_kernel_smem(reinterpret_cast<const void*>(transpose), h->device, adj::TRANSPOSE_SMEM);
+    if (e != cudaSuccess) return e;
+    transpose<<<nb, adj::NT, adj::TRANSPOSE_SMEM, h->stream>>>(
+        h->d_inst, tabs, a, T, phi_n, (const C*)v.M1, (const C*)v.phib, (const C*)v.mub, (const C*)v.uB, lam_next, lam,
+        v.ds);
     h->adj_par ^= 1;
     return cudaGetLastError();
 }

@@ -100,8 +100,8 @@ struct lbch_handle {
     double* h_stage = nullptr;  // pinned host staging
     size_t h_stage_bytes = 0;
     // adjoint workspace (instance 0), allocated by the first lb_ch_adjoint_begin
-    void* adj = nullptr;        // one block: lambda[2] (9N each), mu, grad_mu_bar (2N), F_bar (2N), phi_bar,
-                                // mu_bar, D_bar, u_bar (2N) in the adjoint type; then ds (N) and dL/ds, double
+    void* adj = nullptr;        // one block: lambda[2] (9N each, N at tau_g = 1), M1 (2N), phi_bar, mu_bar, u.B (AdjView);
+                                // then ds (N) and dL/ds, double
     size_t adj_elem = 8;
     int adj_par = 0;            // which lambda holds the current adjoint
     // coupled Navier-Stokes state (LBCH_VEL_COUPLED): f[2], g[2] ([9][N]) and u, p, mu ([N]), one block
