@@ -174,7 +174,7 @@ lbch_status lb_ch_halo_import(lbch_handle* h, int side, const void* src);
  * step: the library then reads and writes phi only (the stored populations are left unchanged and are
  * not part of the state), with the same results bit for bit.  Until lb_ch_tune chooses otherwise, the
  * kernel is chosen by the size of the handle's grids: LBCH_F32 handles whose instances are all periodic with tau_g = 1
- * and fit the device in two waves of two-step tiles (up to about 150 K nodes) step two steps per launch with the two-step
+ * and make up to three 32 x 14 tiles per SM (about 200 K nodes) step two steps per launch with the two-step
  * kernel; the tile kernel steps LBCH_F64 handles of up to about 900 K nodes and, where some tau_g != 1, float ones of up
  * to about 75 K; the row sweep steps every other handle, and those with a Model III instance. */
 lbch_status lb_ch_step(lbch_handle* h, long nsteps);
@@ -221,8 +221,8 @@ void* lb_ch_stream(lbch_handle* h);
  * the tile kernel (each tile's stencil fields staged in shared memory; 32x16, 32x8 and 16x8 with 256
  * threads and 32x16 with 768 on the float paths; 32x8 and 16x8 with 256 and 32x8 with 512 for LBCH_F64)
  * and, for handles whose instances are all periodic with tau_g = 1 in LBCH_F32 or LBCH_F64, the two-step
- * kernel (two steps per launch from phi on the tile + 6; 32x16 with 768 threads, 32x14 and 32x16 with
- * 1024 and 32x8 with 512 in LBCH_F32; 32x8 with 512, 16x8 with 256, 16x16 with 512 and 32x14 with 1024
+ * kernel (two steps per launch from phi on the tile + 6; 32x16, 32x14 and 32x8 with 512 threads and 16x8 with
+ * 256 in LBCH_F32; 32x8 with 512, 16x8 with 256, 16x16 with 512 and 32x14 with 1024
  * in LBCH_F64; an odd last step of lb_ch_step then runs the fastest one-step candidate).  lb_ch_tune
  * times every candidate on the handle's own problem through lb_ch_step (as a run steps: CUDA graphs of 64
  * steps) -- one graph of warm-up, then the faster of two runs of `steps` steps rounded up to whole graphs

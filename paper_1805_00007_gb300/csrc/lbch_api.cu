@@ -1074,14 +1074,20 @@ void choose_default(lbch_handle* h, int sms)
         else if (tiles(3) <= sms) { h->force_tile = true; h->shape = 3; }
         return;
     }
-    // tau_g = 1 in float: the two-step kernel on periodic grids up to two waves of its tiles -- 32 x 8 (100^2: 1.9 per
-    // step against the row sweep's 4.0), one of 32 x 14 (256^2: 2.55 against 4.7), two of 32 x 16 (360^2: 4.7 against
-    // 5.5) --, otherwise the row sweep (512^2: 6.2 against 8.9).  The odd last step of a call, and taped steps, take
+    // tau_g = 1 in float: the two-step kernel on periodic grids up to three of its 32 x 14 tiles per SM -- 16 x 8 and 32 x 8
+    // tiles while every SM gets one (100^2: 1.6 per step against the row sweep's 4.0; 160^2: 1.8), 32 x 14 up to two
+    // (256^2: 2.1 against 4.7; 300^2: 3.1), 32 x 16 up to two (360^2: 3.6 against 5.5), 32 x 14 up to three (400^2: 4.7
+    // against 5.6) --, otherwise the row sweep (512^2: 6.2).  The odd last step of a call, and taped steps, take
     // the one-step kernel that is faster there: 16 x 8 tiles up to three per SM (100^2: 2.7 against 4.0).
     if (!pair_ok(h)) return;
     auto pairs = [&](int k) { return h->pr[k].total_tiles; };
-    h->pshape = pairs(3) <= sms ? 3 : pairs(1) <= sms ? 1 : 2;
-    h->pair = pairs(h->pshape) <= 2 * sms;
+    h->pair = true;
+    if (pairs(2) <= sms) h->pshape = 2;
+    else if (pairs(3) <= sms) h->pshape = 3;
+    else if (pairs(1) <= 2 * sms) h->pshape = 1;
+    else if (pairs(0) <= 2 * sms) h->pshape = 0;
+    else if (pairs(1) <= 3 * sms) h->pshape = 1;
+    else h->pair = false;
     if (h->pair && tiles(2) <= 3 * sms) { h->force_tile = true; h->shape = 2; }
 }
 

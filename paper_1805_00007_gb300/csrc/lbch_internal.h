@@ -26,7 +26,7 @@ struct SweepFit { int warps, sms, nw, width, lead; };
 
 // Tile shapes of the two-step kernel (periodic instances, tau_g = 1; f32 and f64 only).
 constexpr int kPairShapes = 4;
-constexpr Shape kPairF[kPairShapes] = {{32, 16, 768}, {32, 14, 1024}, {32, 16, 1024}, {32, 8, 512}};
+constexpr Shape kPairF[kPairShapes] = {{32, 16, 512}, {32, 14, 512}, {16, 8, 256}, {32, 8, 512}};
 constexpr Shape kPair64[kPairShapes] = {{32, 8, 512}, {16, 8, 256}, {16, 16, 512}, {32, 14, 1024}};
 inline Shape pair_shape(int prec, int k) { return prec == LBCH_F64 ? kPair64[k] : kPairF[k]; }
 

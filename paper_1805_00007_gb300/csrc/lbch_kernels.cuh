@@ -481,23 +481,14 @@ __device__ __forceinline__ void store_h(C* H, long long plane, int row0, int pit
     }
 }
 
-// The nodes of a W x H region that the CTA's NT threads take in one phase: f(e, r, c) for node e = r W + c.
-// STRIDE = W: consecutive threads take consecutive nodes.  STRIDE = W + 2, the row width of the region the
-// phase reads its stencil operands from: thread index i stands for row i / STRIDE and column i % STRIDE, and
-// the two columns past W idle.  A warp's operand reads then cover consecutive words of the source region;
-// with the compact order a warp that crosses a row boundary spans STRIDE + 2 words, so that two of its reads
-// fall in one shared-memory bank.  The wider order is taken only where it needs no more passes of the NT
-// threads than the compact one, and only where the step is bound by latency rather than a pipe: the FP64
-// kernels are bound by the FP64 pipe, where a warp's idle lanes still take their pipe slots (the FP64 tile
-// kernel ran 6 % slower with it).  The two-step kernel in float uses it.
-template <int W, int H, int STRIDE, int NT, typename F>
+// The nodes of a W x H region that the CTA's NT threads take in one phase, consecutive threads consecutive nodes:
+// f(e, r, c) for node e = r W + c.
+template <int W, int H, int NT, typename F>
 __device__ __forceinline__ void for_region(F&& f)
 {
-    constexpr int SW = (H * STRIDE + NT - 1) / NT == (H * W + NT - 1) / NT ? STRIDE : W;
-    for (int i = threadIdx.x; i < H * SW; i += NT) {
-        const int r = i / SW, c = i - r * SW;
-        if (SW != W && c >= W) continue;
-        f(r * W + c, r, c);
+    for (int i = threadIdx.x; i < H * W; i += NT) {
+        const int r = i / W;
+        f(i, r, i - r * W);
     }
 }
 
@@ -641,7 +632,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         }
         // the counter is read only when the launch needs the step index; otherwise nothing waits on that load
         s_time = a.read_n ? a.ctl->time : 0;
-        if (s_tile_inst >= 0) s_T = (C)step_T(a.Tf, s_tile_inst, s_I, s_time + a.t_off);
+        if (s_tile_inst >= 0) s_T = a.need_time ? (C)step_T(a.Tf, s_tile_inst, s_I, s_time + a.t_off) : C(1);
     }
     __syncthreads();
     const long long n = s_time + a.t_off;
@@ -667,7 +658,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
             if (tid == 0) {
                 s_I = a.inst[cur_inst];
                 s_tile_inst = cur_inst;
-                s_T = (C)step_T(a.Tf, cur_inst, s_I, n);  // time factor of the flow, once per instance
+                s_T = a.need_time ? (C)step_T(a.Tf, cur_inst, s_I, n) : C(1);  // time factor of the flow, once per instance
             }
             __syncthreads();
         }
@@ -706,7 +697,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         C* s_z = s_mu + L::OFF_COLS / sizeof(C);
         if constexpr (L::COLS) {
             constexpr int AW = L::AW, AN = L::AN;
-            for_region<AW, MH, AW, NT>([&](int e, int r, int c) {
+            for_region<AW, MH, NT>([&](int e, int r, int c) {
                 const P* q = pb + (r + 1) * BW + c + 1;
                 const C pS = cvt<C>(q[-BW]), ce = cvt<C>(q[0]), pN = cvt<C>(q[BW]);
                 C dl;
@@ -721,15 +712,13 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
                 }
             });
             __syncthreads();
-            for_region<MW, L::MH, MW, NT>([&](int e, int r, int c) {
+            for_region<MW, L::MH, NT>([&](int e, int r, int c) {
                 const int k = r * AW + c + 1;
                 s_mu[e] = node_mu(cvt<C>(pb[(r + 1) * BW + c + 2]), s_z[AN + k], s_z[k], s_z[k + 1], s_z[k - 1], K0);
                 if (model >= 2) s_D[e] = node_div(s_z[2 * AN + k], s_z[3 * AN + k + 1], s_z[4 * AN + k - 1]);
             });
         } else
-        // (the compact order in every phase: the strided order of for_region measured no faster here, 4.56
-        // against 4.55 us per step for 256^2 at tau_g = 0.8 in FP32, 4.30 against 4.23 with half storage)
-        for_region<MW, L::MH, MW, NT>([&](int e, int r, int c) {
+        for_region<MW, L::MH, NT>([&](int e, int r, int c) {
             const P* q = pb + (r + 1) * BW + c + 2;
             C ce = cvt<C>(q[0]);
             C pE = cvt<C>(q[1]), pW = cvt<C>(q[-1]), pN = cvt<C>(q[BW]), pS = cvt<C>(q[-BW]);
@@ -760,7 +749,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         // the column values of mu and D (in the place of phi's)
         constexpr int CN = MW * L::GH;
         if constexpr (L::COLS) {
-            for_region<MW, L::GH, MW, NT>([&](int e, int r, int c) {
+            for_region<MW, L::GH, NT>([&](int e, int r, int c) {
                 const C mS = s_mu[e], mN = s_mu[e + 2 * MW];
                 s_z[e] = node_w(mS, s_mu[e + MW], mN);
                 s_z[CN + e] = mN - mS;
@@ -774,7 +763,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         }
 
         // 3. force, equilibrium, source and collision on tile + 1, written back into the box
-        for_region<GW, L::GH, GW, NT>([&](int e, int r, int c) {
+        for_region<GW, L::GH, NT>([&](int e, int r, int c) {
             int gy = y0 - 1 + r;
             if (walls && (gy < 0 || gy >= ny)) return;  // ghost rows: never pulled (bounce-back)
             int m = (r + 1) * MW + (c + 1);
@@ -847,7 +836,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         //    Interior nodes (no wall neighbour, no ghost image) take a straight path without the checks.
         const int pitch = a.pitch;
         const float* lb = reinterpret_cast<const float*>(stage(s) + L::OFF_L);
-        for_region<TX, TY, TX, NT>([&](int e, int r, int c) {
+        for_region<TX, TY, NT>([&](int e, int r, int c) {
             int gx = x0 + c, gy = y0 + r;
             if (gx >= nx || gy >= ny) return;
             const bool wallrow = walls && (gy == 0 || gy == ny - 1);

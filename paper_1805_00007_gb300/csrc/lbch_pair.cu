@@ -74,9 +74,9 @@ cudaError_t lbch_launch_pair(lbch_handle* h, int parity)
         return k == 0 ? launch_pair_v<double, double, 32, 8, 512>(h, parity)
              : k == 1 ? launch_pair_v<double, double, 16, 8, 256>(h, parity)
              : k == 2 ? launch_pair_v<double, double, 16, 16, 512>(h, parity) : launch_pair_v<double, double, 32, 14, 1024>(h, parity);
-    return k == 0 ? launch_pair_v<float, float, 32, 16, 768>(h, parity)
-         : k == 1 ? launch_pair_v<float, float, 32, 14, 1024>(h, parity)
-         : k == 2 ? launch_pair_v<float, float, 32, 16, 1024>(h, parity) : launch_pair_v<float, float, 32, 8, 512>(h, parity);
+    return k == 0 ? launch_pair_v<float, float, 32, 16, 512>(h, parity)
+         : k == 1 ? launch_pair_v<float, float, 32, 14, 512>(h, parity)
+         : k == 2 ? launch_pair_v<float, float, 16, 8, 256>(h, parity) : launch_pair_v<float, float, 32, 8, 512>(h, parity);
 }
 
 cudaError_t lbch_prepare_pair(lbch_handle* h, int k)
@@ -86,7 +86,7 @@ cudaError_t lbch_prepare_pair(lbch_handle* h, int k)
         return k == 0 ? prepare_pair_v<double, double, 32, 8, 512>(h, k)
              : k == 1 ? prepare_pair_v<double, double, 16, 8, 256>(h, k)
              : k == 2 ? prepare_pair_v<double, double, 16, 16, 512>(h, k) : prepare_pair_v<double, double, 32, 14, 1024>(h, k);
-    return k == 0 ? prepare_pair_v<float, float, 32, 16, 768>(h, k)
-         : k == 1 ? prepare_pair_v<float, float, 32, 14, 1024>(h, k)
-         : k == 2 ? prepare_pair_v<float, float, 32, 16, 1024>(h, k) : prepare_pair_v<float, float, 32, 8, 512>(h, k);
+    return k == 0 ? prepare_pair_v<float, float, 32, 16, 512>(h, k)
+         : k == 1 ? prepare_pair_v<float, float, 32, 14, 512>(h, k)
+         : k == 2 ? prepare_pair_v<float, float, 16, 8, 256>(h, k) : prepare_pair_v<float, float, 32, 8, 512>(h, k);
 }

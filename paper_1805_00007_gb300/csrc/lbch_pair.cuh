@@ -83,7 +83,7 @@ template <typename C, typename P, int W, int H, int PW, int NT>
 __device__ __forceinline__ void pair_mu_div(const P* ph, const C* sX1, const C* sX2, const C* sY1, const C* sY2,
                                             int to, const Consts<C>& K0, bool model2, C* s_mu, C* s_D)
 {
-    for_region<W, H, sizeof(C) == 4 ? PW : W, NT>([&](int e, int r, int c) {
+    for_region<W, H, NT>([&](int e, int r, int c) {
         const P* q = ph + (r + 1) * PW + c + 1;
         const C ce = cvt<C>(q[0]);
         const C pE = cvt<C>(q[1]), pW = cvt<C>(q[-1]), pN = cvt<C>(q[PW]), pS = cvt<C>(q[-PW]);
@@ -106,7 +106,7 @@ __device__ __forceinline__ void pair_collide(const P* ph_reg, const C* s_mu, con
                                              const C* sX2, const C* sY1, const C* sY2, int tu, const Consts<C>& K0,
                                              bool model2, C* s_post)
 {
-    for_region<W, H, sizeof(C) == 4 ? MW : W, NT>([&](int e, int r, int c) {
+    for_region<W, H, NT>([&](int e, int r, int c) {
         const int m = (r + 1) * MW + (c + 1);
         C gmx, gmy, gDx = C(0), gDy = C(0);
         grad9(s_mu[m + 1], s_mu[m - 1], s_mu[m + MW], s_mu[m - MW], s_mu[m + MW + 1], s_mu[m + MW - 1],
@@ -139,6 +139,112 @@ __device__ __forceinline__ C pair_pull(const C* s_post, int r, int c, C& v0)
 #pragma unroll
     for (int q = 1; q < 9; q++) v[q] = s_post[q * NP + p - cy(q) * PW - cx(q)];
     return stream_sum_q(v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8]);
+}
+
+// ---- the same phases with two neighbouring nodes per thread (the float path)
+//
+// In float the launch is bound by latency and instruction issue.  A thread that takes the pair (a, b) of a row loads the
+// neighbourhood of both as aligned pairs of values (15 loads instead of 38 for mu and D, 17 instead of 44 for the
+// collision, 12 instead of 18 for the pull), forms the column values they share once, and halves the index arithmetic,
+// with the values and operations of the one-node phases (600 instructions per update instead of 780).  Half the threads
+// take every phase of a 32 x 14 tile in one pass, and at 64 registers two blocks of 512 fit on an SM, so that a launch's
+// blocks set up (tables, load offsets) beside the previous launch's last phases.  Us per step before -> with pairs ->
+// with two blocks per SM: 256^2 2.55 -> 2.56 -> 2.10; 100^2 1.90 (32 x 8) -> 1.84 -> 1.56 (16 x 8); 360^2 4.7 -> 4.6 -> 3.6.
+template <int W, int H, int NT, typename F> __device__ __forceinline__ void for_pairs(F&& f)
+{
+    static_assert(W % 2 == 0, "whole pairs");
+    for (int i = threadIdx.x; i < H * (W / 2); i += NT) {
+        const int r = i / (W / 2);
+        f(r, 2 * (i - r * (W / 2)));
+    }
+}
+__device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ void st2(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
+// four neighbouring values from an even offset
+struct Quad { float L, a, b, R; };
+__device__ __forceinline__ Quad ld4(const float* p)
+{
+    const float2 u = ld2(p), v = ld2(p + 2);
+    return {u.x, u.y, v.x, v.y};
+}
+
+template <int W, int H, int PW, int NT>
+__device__ __forceinline__ void pair_mu_div2(const float* ph, const float* sX1, const float* sX2, const float* sY1,
+                                             const float* sY2, int to, const Consts<float>& K0, bool model2, float* s_mu,
+                                             float* s_D)
+{
+    for_pairs<W, H, NT>([&](int r, int c) {
+        const float* q = ph + r * PW + c;
+        const Quad S = ld4(q), M = ld4(q + PW), N = ld4(q + 2 * PW);
+        float dl, dla, dlb;
+        const float zL = node_z(S.L, M.L, N.L, dl), za = node_z(S.a, M.a, N.a, dla);
+        const float zb = node_z(S.b, M.b, N.b, dlb), zR = node_z(S.R, M.R, N.R, dl);
+        st2(s_mu + r * W + c, node_mu(M.a, dla, za, zb, zL, K0), node_mu(M.b, dlb, zb, zR, za, K0));
+        if (model2) {
+            const float *x1 = sX1 + c + to, *x2 = sX2 + c + to, *y1 = sY1 + r + to, *y2 = sY2 + r + to;
+            const float y1S = y1[0], y14 = op_mul(4.0f, y1[1]), y1N = y1[2], y2S = y2[0], y2N = y2[2];
+            float E, Ea, Eb, ER, WL, Wa, Wb, W_;
+            node_flux(S.L, M.L, N.L, x1[0], x2[0], y1S, y14, y1N, y2S, y2N, E, WL);
+            const float da = node_flux(S.a, M.a, N.a, x1[1], x2[1], y1S, y14, y1N, y2S, y2N, Ea, Wa);
+            const float db = node_flux(S.b, M.b, N.b, x1[2], x2[2], y1S, y14, y1N, y2S, y2N, Eb, Wb);
+            node_flux(S.R, M.R, N.R, x1[3], x2[3], y1S, y14, y1N, y2S, y2N, ER, W_);
+            st2(s_D + r * W + c, node_div(da, Eb, WL), node_div(db, ER, Wa));
+        }
+    });
+}
+
+// 12 grad of a field at the pair from its values on the region one node wider (row stride MW), q at the south-west
+template <int MW>
+__device__ __forceinline__ void grad_pair(const float* q, float2& gx, float2& gy, float2& mid)
+{
+    const Quad S = ld4(q), M = ld4(q + MW), N = ld4(q + 2 * MW);
+    const float wL = node_w(S.L, M.L, N.L), wa = node_w(S.a, M.a, N.a), wb = node_w(S.b, M.b, N.b), wR = node_w(S.R, M.R, N.R);
+    const float da = N.a - S.a, db = N.b - S.b;
+    gx = make_float2(wb - wL, wR - wa);
+    gy = make_float2(node_gy(N.L - S.L, da, db), node_gy(da, db, N.R - S.R));
+    mid = make_float2(M.a, M.b);
+}
+
+template <int W, int H, int MW, int PW, int NT>
+__device__ __forceinline__ void pair_collide2(const float* ph_reg, const float* s_mu, const float* s_D, const float* sX1,
+                                              const float* sX2, const float* sY1, const float* sY2, int tu,
+                                              const Consts<float>& K0, bool model2, float* s_post)
+{
+    for_pairs<W, H, NT>([&](int r, int c) {
+        float2 gmx, gmy, gDx = make_float2(0.0f, 0.0f), gDy = gDx, mu, D;
+        grad_pair<MW>(s_mu + r * MW + c, gmx, gmy, mu);
+        if (model2) grad_pair<MW>(s_D + r * MW + c, gDx, gDy, D);
+        const float2 ph = ld2(ph_reg + (r + 2) * PW + c + 2);
+        const float y1 = sY1[r + tu], y2 = sY2[r + tu];
+        auto node = [&](float p, float m, float gx, float gy, float dx, float dy, int k, float* post) {
+            const float ux = node_u(sX1[c + tu + k], y1), uy = node_u(sX2[c + tu + k], y2);
+            float Px, Py, Jx, Jy;
+            node_flow(p, ux, uy, K0, Px, Py);
+            node_force(p, gx, gy, dx, dy, Px, Py, model2, K0, Jx, Jy);
+            collide9<float, true>(m, ux, uy, Px, Py, Jx, Jy, nullptr, K0, post);
+        };
+        float pa[9], pb[9];
+        node(ph.x, mu.x, gmx.x, gmy.x, gDx.x, gDy.x, 0, pa);
+        node(ph.y, mu.y, gmx.y, gmy.y, gDx.y, gDy.y, 1, pb);
+#pragma unroll
+        for (int q = 0; q < 9; q++) st2(s_post + q * (W * H) + r * W + c, pa[q], pb[q]);
+    });
+}
+
+// The streamed populations at the pair (r, c), (r, c + 1) of a region of width W: what comes from the columns to either
+// side lies at even offsets of the region one node wider, what stays in its column at odd ones.
+template <int W, int NP>
+__device__ __forceinline__ float2 pair_pull2(const float* s_post, int r, int c, float2& v0)
+{
+    constexpr int PW = W + 2;
+    const float* p = s_post + r * PW + c;
+    const float2 v1 = ld2(p + 1 * NP + PW), v5 = ld2(p + 5 * NP), v8 = ld2(p + 8 * NP + 2 * PW);
+    const float2 v3 = ld2(p + 3 * NP + PW + 2), v6 = ld2(p + 6 * NP + 2), v7 = ld2(p + 7 * NP + 2 * PW + 2);
+    const float* p2 = p + 2 * NP + 1;
+    const float* p4 = p + 4 * NP + 2 * PW + 1;
+    v0 = make_float2(p[PW + 1], p[PW + 2]);
+    return make_float2(stream_sum_q(v1.x, p2[0], v3.x, p4[0], v5.x, v6.x, v7.x, v8.x),
+                       stream_sum_q(v1.y, p2[1], v3.y, p4[1], v5.y, v6.y, v7.y, v8.y));
 }
 
 // phi(t+1) = phi(t) + g_0 + sum_q g_q on the float path: hi + lo absorbs the increment exactly (TwoSum),
@@ -272,12 +378,75 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
         Yb2 = Yb1 + L::H6;
     }
 
+    const int nx = I.nx, ny = I.ny;
+    // phi(t+2) of a domain node, with its periodic images in the ghost frame (three deep), read by one-step launches
+    auto images = [&](int gx, int gy, P hi) {
+        if (gx >= 3 && gx < nx - 3 && gy >= 3 && gy < ny - 3) return;
+        const int xa = gx < 3 ? gx + nx : NONE, xb = gx >= nx - 3 ? gx - nx : NONE;
+        const int ya = gy < 3 ? gy + ny : NONE, yb = gy >= ny - 3 ? gy - ny : NONE;
+        for (int iy = 0; iy < 3; iy++) {
+            const int yy = iy == 0 ? gy : (iy == 1 ? ya : yb);
+            if (yy == NONE) continue;
+            for (int ix = 0; ix < 3; ix++) {
+                const int xx = ix == 0 ? gx : (ix == 1 ? xa : xb);
+                if (xx == NONE || (ix == 0 && iy == 0)) continue;
+                phi_out[rb + (long long)yy * pitch + xx] = hi;
+            }
+        }
+    };
+
+    if constexpr (kFF) {
+        // step t: mu, D on tile + 5; collision on tile + 4; streaming to phi(t+1) on tile + 3
+        pair_mu_div2<L::W5, L::H5, W6, NT>(S.phi0, S.X1, S.X2, Ya1, Ya2, 0, K0, model2, S.mu, S.D);
+        __syncthreads();
+        pair_collide2<L::W4, L::H4, L::W5, W6, NT>(S.phi0, S.mu, S.D, S.X1, S.X2, Ya1, Ya2, 2, K0, model2, S.post);
+        __syncthreads();
+        for_pairs<W3, L::H3, NT>([&](int r, int c) {
+            float2 v0;
+            const float2 sum = pair_pull2<W3, L::N4>(S.post, r, c, v0);
+            const float* h = S.phi0 + (r + 3) * W6 + c + 3;
+            const float2 l = ld2(S.lo0 + r * W3 + c);
+            float la, lb;
+            const float ha = pair_phi<C, P, kFF>(h[0], l.x, v0.x, sum.x, la), hb = pair_phi<C, P, kFF>(h[1], l.y, v0.y, sum.y, lb);
+            st2(S.hi1 + r * W3 + c, ha, hb);
+            st2(S.lo1 + r * W3 + c, la, lb);
+        });
+        __syncthreads();
+
+        // step t+1: mu, D on tile + 2; collision on tile + 1; streaming to phi(t+2) on the tile
+        pair_mu_div2<L::W2, L::H2, W3, NT>(S.hi1, S.X1, S.X2, Yb1, Yb2, 3, K0, model2, S.mu, S.D);
+        __syncthreads();
+        pair_collide2<L::W1, L::H1, L::W2, W3, NT>(S.hi1, S.mu, S.D, S.X1, S.X2, Yb1, Yb2, 5, K0, model2, S.post);
+        __syncthreads();
+        for_pairs<TX, TY, NT>([&](int r, int c) {
+            const int gx = x0 + c, gy = y0 + r;
+            if (gx >= nx || gy >= ny) return;
+            float2 v0;
+            const float2 sum = pair_pull2<TX, L::N1>(S.post, r, c, v0);
+            const int k = (r + 3) * W3 + c + 3;
+            float la, lb;
+            const float ha = pair_phi<C, P, kFF>(S.hi1[k], S.lo1[k], v0.x, sum.x, la);
+            const float hb = pair_phi<C, P, kFF>(S.hi1[k + 1], S.lo1[k + 1], v0.y, sum.y, lb);
+            const long long node = rb + (long long)gy * pitch + gx;
+            if (gx + 1 < nx) {
+                st2(phi_out + node, ha, hb);
+                st2(lo_out + node, la, lb);
+            } else {
+                phi_out[node] = ha;
+                lo_out[node] = la;
+            }
+            images(gx, gy, ha);
+            if (gx + 1 < nx) images(gx + 1, gy, hb);
+        });
+        return;
+    }
+
     // step t: mu, D on tile + 5; collision on tile + 4; streaming to phi(t+1) on tile + 3
     pair_mu_div<C, P, L::W5, L::H5, W6, NT>(S.phi0, S.X1, S.X2, Ya1, Ya2, 0, K0, model2, S.mu, S.D);
     __syncthreads();
     pair_collide<C, P, L::W4, L::H4, L::W5, W6, NT, kShift>(S.phi0, S.mu, S.D, S.X1, S.X2, Ya1, Ya2, 2, K0, model2, S.post);
     __syncthreads();
-    for_region<W3, L::H3, sizeof(C) == 4 ? L::W4 : W3, NT>([&](int e, int r, int c) {
+    for_region<W3, L::H3, NT>([&](int e, int r, int c) {
         C v0;
         const C sumq = pair_pull<C, W3, L::N4>(S.post, r, c, v0);
         float lo1;
@@ -291,8 +460,7 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
     __syncthreads();
     pair_collide<C, P, L::W1, L::H1, L::W2, W3, NT, kShift>(S.hi1, S.mu, S.D, S.X1, S.X2, Yb1, Yb2, 5, K0, model2, S.post);
     __syncthreads();
-    const int nx = I.nx, ny = I.ny;
-    for_region<TX, TY, sizeof(C) == 4 ? L::W1 : TX, NT>([&](int e, int r, int c) {
+    for_region<TX, TY, NT>([&](int e, int r, int c) {
         const int gx = x0 + c, gy = y0 + r;
         if (gx >= nx || gy >= ny) return;
         C v0;
@@ -303,20 +471,7 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
         const long long node = rb + (long long)gy * pitch + gx;
         phi_out[node] = hi;
         if (kFF) lo_out[node] = lo;
-        if (gx < 3 || gx >= nx - 3 || gy < 3 || gy >= ny - 3) {
-            // the node's periodic images in the ghost frame (three deep), read by one-step launches
-            const int xa = gx < 3 ? gx + nx : NONE, xb = gx >= nx - 3 ? gx - nx : NONE;
-            const int ya = gy < 3 ? gy + ny : NONE, yb = gy >= ny - 3 ? gy - ny : NONE;
-            for (int iy = 0; iy < 3; iy++) {
-                const int yy = iy == 0 ? gy : (iy == 1 ? ya : yb);
-                if (yy == NONE) continue;
-                for (int ix = 0; ix < 3; ix++) {
-                    const int xx = ix == 0 ? gx : (ix == 1 ? xa : xb);
-                    if (xx == NONE || (ix == 0 && iy == 0)) continue;
-                    phi_out[rb + (long long)yy * pitch + xx] = hi;
-                }
-            }
-        }
+        images(gx, gy, hi);
     });
 }
 
@@ -337,7 +492,7 @@ __device__ __forceinline__ void pair_locate(const int* tile_begin, int n_inst, c
 // memory round trip (the table loads start at once, the phi loads right after the dependency wait), and the
 // per-node helpers take the instance's constants as constant-bank operands instead of loading them.
 template <typename C, typename P, int TX, int TY, int NT, bool SINGLE>
-__global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __grid_constant__ PairArgs<C, P> a)
+__global__ void __launch_bounds__(NT, NT > 512 ? 1 : 2) ch_pair_kernel(const __grid_constant__ PairArgs<C, P> a)
 {
     extern __shared__ unsigned char smem_raw[];
     const PairSmem<C, P, TX, TY> S(smem_raw);
@@ -383,8 +538,10 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __
         if (tid == 0) {
             if (any) wait_tables();
             s_time = a.read_n ? a.ctl->time : 0;
-            s_T[0] = (C)step_T(a.Tf, 0, I, s_time + a.t_off);
-            s_T[1] = (C)step_T(a.Tf, 1, I, s_time + a.t_off + 1);
+            if (a.need_time) {  // (forming the 1 of a steady flow takes its thread 0.2 us of the launch)
+                s_T[0] = (C)step_T(a.Tf, 0, I, s_time + a.t_off);
+                s_T[1] = (C)step_T(a.Tf, 1, I, s_time + a.t_off + 1);
+            }
         }
         __syncthreads();
         n = s_time + a.t_off;
@@ -428,7 +585,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __
         if (tid == 0) {
             if (any) wait_tables();
             s_time = a.read_n ? a.ctl->time : 0;
-            if (s_k >= 0) {
+            if (s_k >= 0 && a.need_time) {
                 s_T[0] = (C)step_T(a.Tf, s_k, s_I, s_time + a.t_off);
                 s_T[1] = (C)step_T(a.Tf, a.n_inst + s_k, s_I, s_time + a.t_off + 1);
             }
@@ -440,7 +597,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) ch_pair_kernel(const __
                 __syncthreads();  // the previous tile's shared data are read no more
                 if (tid == 0) {
                     pair_fetch_tables<C, P, TX, TY>(S, a.ttabs, t, &s_tbar);
-                    if (locate(t)) {
+                    if (locate(t) && a.need_time) {
                         s_T[0] = (C)step_T(a.Tf, s_k, s_I, n);
                         s_T[1] = (C)step_T(a.Tf, a.n_inst + s_k, s_I, n + 1);
                     }

@@ -58,6 +58,7 @@ struct SweepArgs {
     Ctl* ctl;
     int t_off;              // this launch's step is ctl->time + t_off
     int t_adv;              // when nonzero, the launch's last CTA advances ctl->time by t_adv
+    int timed;              // some instance's flow has a time factor
     int read_n;             // the launch reads the step index: Model III, or a time factor without a table
     const double* Tf;       // the instances' time factors at this launch's step, or null (step_T)
     const S* g_in;          // populations (GEN): g[(row * nq + plane) * pitch + column]
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(SweepShape<S, P, FF, GEN, GEN && (WALLS || !SI
     grid_dependency_wait();
     grid_launch_dependents();
     const long long n = a.read_n ? a.ctl->time + a.t_off : 0;
-    const C T = (C)step_T(a.Tf, k_t, I, n);
+    const C T = a.timed ? (C)step_T(a.Tf, k_t, I, n) : C(1);
 
     if (mine) {
         const bool model2 = M3 ? I.model >= 2 : I.model == 2;  // D = div(phi u) is needed (Models II, III)

@@ -27,6 +27,7 @@ cudaError_t launch_sweep_v(lbch_handle* h, int parity)
     a.ctl = h->ctl;
     a.t_off = h->t_off;
     a.t_adv = h->t_adv;
+    a.timed = h->timed;
     a.Tf = launch_T(h);
     a.read_n = launch_reads_n(h);
     a.g_in = static_cast<const S*>(h->g[parity]);
