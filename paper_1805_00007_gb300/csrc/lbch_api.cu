@@ -355,20 +355,18 @@ template <typename C>
 ns::NsArgs<C> ns_args(lbch_handle* h, int parity)
 {
     const InstDev& I = h->inst[0];
-    const size_t N = (size_t)I.nx * I.ny;
     ns::NsArgs<C> a;
     a.nx = I.nx; a.ny = I.ny; a.walls = I.walls; a.model = I.model; a.pitch = h->pitch; a.row0 = I.row0;
+    a.nb = ns::groups_of(I.nx);
     a.k = ch_consts<C>(I);
     a.n = ns_consts<C>(h);
     C* p = static_cast<C*>(h->ns);
-    C* f[2] = {p, p + 9 * N};
-    C* g[2] = {p + 18 * N, p + 27 * N};
-    a.f_in = f[parity]; a.f_out = f[parity ^ 1];
-    a.g_in = g[parity]; a.g_out = g[parity ^ 1];
-    C* w = p + 36 * N;
-    a.ux = w; a.uy = w + N; a.pr = w + 2 * N; a.mu = w + 3 * N;
-    a.phi_in = static_cast<C*>(h->phi[parity]);
-    a.phi_out = static_cast<C*>(h->phi[parity ^ 1]);
+    const size_t S = ns::state_elems(I.nx, I.ny);
+    a.in = p + (parity ? S : 0);
+    a.out = p + (parity ? 0 : S);
+    a.aux = p + 2 * S;
+    a.phi = static_cast<C*>(h->phi[parity]);
+    a.obs = a.out;  // the next state's buffer, which the next step fills completely
     return a;
 }
 
@@ -378,10 +376,19 @@ template <typename C>
 cudaError_t launch_ns_t(lbch_handle* h, int parity)
 {
     ns::NsArgs<C> a = ns_args<C>(h, parity);
-    const int tiles = ns::tiles_of(a.nx, a.ny);
-    ns::fields_kernel<C><<<tiles, ns::NT, 0, h->stream>>>(a);
-    ns::collide_kernel<C><<<tiles, ns::NTC, 0, h->stream>>>(a);
-    return cudaGetLastError();
+    // each kernel a programmatic dependent of the one before it in the stream
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ns::tiles_of(a.nx, a.ny));
+    cfg.blockDim = dim3(ns::NT);
+    cfg.stream = h->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = h->no_pdl ? 0 : 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaError_t e = cudaLaunchKernelEx(&cfg, ns::fields_kernel<C, false>, a)) return e;
+    const bool one = a.k.omt == C(0) && !h->force_general;
+    return cudaLaunchKernelEx(&cfg, one ? ns::collide_kernel<C, true> : ns::collide_kernel<C, false>, a);
 }
 
 // phi of the current state of a coupled handle into its phi array (the steps leave it to the next step).
@@ -405,7 +412,7 @@ template <typename C>
 cudaError_t ns_fields_t(lbch_handle* h, int parity)
 {
     ns::NsArgs<C> a = ns_args<C>(h, parity);
-    ns::fields_kernel<C><<<ns::tiles_of(a.nx, a.ny), ns::NT, 0, h->stream>>>(a);
+    ns::fields_kernel<C, true><<<ns::tiles_of(a.nx, a.ny), ns::NT, 0, h->stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -1347,14 +1354,17 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
         h->nsd.itauf = 1.0 / h->nsd.tauf; h->nsd.omtf = 1.0 - h->nsd.itauf; h->nsd.srcf = 1.0 - 0.5 / h->nsd.tauf;
         h->nsf.itauf = (float)h->nsd.itauf; h->nsf.omtf = (float)h->nsd.omtf; h->nsf.srcf = (float)h->nsd.srcf;
         const size_t N = (size_t)d.nx * d.ny, esz = prec == LBCH_F64 ? 8 : 4;
-        CKI(dalloc(h, &h->ns, 40 * N * esz));  // f, g (two buffers each), u, p, mu
-        CKI(cudaMemsetAsync(h->ns, 0, 40 * N * esz, h->stream));
+        const size_t bytes = (2 * ns::state_elems(d.nx, d.ny) + ns::aux_elems(d.nx, d.ny)) * esz;
+        CKI(dalloc(h, &h->ns, bytes));  // g and f (two states) and the fields between the kernels
+        CKI(cudaMemsetAsync(h->ns, 0, bytes, h->stream));
         const int nbn = (int)((N + 255) / 256);
         if (prec == LBCH_F64) {
-            ns::NsArgs<double> a = ns_args<double>(h, 1);  // writes the parity-0 buffers
+            ns::NsArgs<double> a = ns_args<double>(h, 1);  // writes the parity-0 state
+            a.phi = static_cast<double*>(h->phi[0]);
             ns::init_kernel<double><<<nbn, 256, 0, h->stream>>>(a, h->phi0);
         } else {
             ns::NsArgs<float> a = ns_args<float>(h, 1);
+            a.phi = static_cast<float*>(h->phi[0]);
             ns::init_kernel<float><<<nbn, 256, 0, h->stream>>>(a, h->phi0);
         }
         CKI(cudaGetLastError());
@@ -1512,7 +1522,8 @@ lbch_status lb_ch_observe(lbch_handle* h, int inst, int what, double* out)
         const size_t N = (size_t)h->inst[0].nx * h->inst[0].ny, e = h->prec == LBCH_F64 ? 8 : 4;
         lbch_status s = stage(h, 2 * N * sizeof(double));
         if (s != LBCH_OK) return s;
-        const char* w = static_cast<const char*>(h->ns) + 36 * N * e;  // ux, uy, pr, mu
+        const InstDev& d = h->inst[0];
+        const char* w = static_cast<const char*>(h->ns) + (parity ? 0 : ns::state_elems(d.nx, d.ny) * e);  // u, p (NsArgs::obs)
         if (what == LBCH_OBS_U) CK(cudaMemcpyAsync(h->h_stage, w, 2 * N * e, cudaMemcpyDeviceToHost, h->stream));
         else CK(cudaMemcpyAsync(h->h_stage, w + 2 * N * e, N * e, cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
@@ -1969,11 +1980,10 @@ lbch_status lb_ch_test_hook(lbch_handle* h, int hook, long value)
         const int nxt = cur_buf(h) ^ 1;
         if (h->coupled) {
             const InstDev& d = h->inst[0];
-            const size_t N = (size_t)d.nx * d.ny, e = h->prec == LBCH_F64 ? 8 : 4;
+            const size_t e = h->prec == LBCH_F64 ? 8 : 4, S = ns::state_elems(d.nx, d.ny) * e;
             char* p = static_cast<char*>(h->ns);
-            CK(cudaMemsetAsync(p + (size_t)nxt * 9 * N * e, 0xFF, 9 * N * e, h->stream));         // f
-            CK(cudaMemsetAsync(p + (18 + (size_t)nxt * 9) * N * e, 0xFF, 9 * N * e, h->stream));  // g
-            CK(cudaMemsetAsync(p + 36 * N * e, 0xFF, 4 * N * e, h->stream));                      // u, p, mu
+            CK(cudaMemsetAsync(p + (nxt ? S : 0), 0xFF, S, h->stream));                                // g, f
+            CK(cudaMemsetAsync(p + 2 * S, 0xFF, ns::aux_elems(d.nx, d.ny) * e, h->stream));            // phi, u, mu, p
             // phi of the current state: the next step forms it from the populations before reading it
             CK(cudaMemsetAsync(h->phi[nxt ^ 1], 0xFF, (size_t)h->rows * h->pitch * h->phi_elem, h->stream));
         } else {
