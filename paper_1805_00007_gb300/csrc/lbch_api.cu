@@ -367,6 +367,7 @@ ns::NsArgs<C> ns_args(lbch_handle* h, int parity)
     a.aux = p + 2 * S;
     a.phi = static_cast<C*>(h->phi[parity]);
     a.obs = a.out;  // the next state's buffer, which the next step fills completely
+    ns::set_folded(a);
     return a;
 }
 
