@@ -82,7 +82,6 @@ struct lbch_handle {
     double* phi0 = nullptr;     // initial field, double, padded layout
     lbch::Ctl* ctl = nullptr;
     double* partials = nullptr; // reduction scratch: n_inst * chunks * RED_NV doubles
-    double* result = nullptr;   // n_inst * RED_NV doubles
     int chunks = 0;
     long long n = 0;            // host mirror of the step index
     int flip = 0;               // the state of step n is in buffer (n & 1) ^ flip (two-step launches toggle it)

@@ -1070,7 +1070,7 @@ __global__ void __launch_bounds__(RED_NT) reduce_partials_kernel(const InstDev* 
     const long long N = (long long)I.nx * I.ny;
     double v[RED_NV] = {0.0, 0.0, 0.0, -INFINITY, INFINITY, 0.0};
     for (long long k = (long long)blockIdx.x * RED_NT + threadIdx.x; k < N; k += (long long)chunks * RED_NT) {
-        int y = (int)(k / I.nx), x = (int)(k - (long long)y * I.nx);
+        const int y = N <= 0x7fffffffLL ? (int)((unsigned)k / (unsigned)I.nx) : (int)(k / I.nx), x = (int)(k - (long long)y * I.nx);
         long long gi = (long long)(I.row0 + y) * pitch + GC + x;
         double p = (double)phi[gi] + (lo ? (double)lo[gi] : 0.0), p0 = phi0[gi];
         if (!isfinite(p)) { v[5] += 1.0; continue; }
@@ -1085,7 +1085,10 @@ __global__ void __launch_bounds__(RED_NT) reduce_partials_kernel(const InstDev* 
     }
 }
 
-static __global__ void __launch_bounds__(RED_NT) reduce_final_kernel(const double* partials, int chunks, double* result)
+// The sums of an instance, and after those of all instances the error flags of the steps, into pinned host memory: the
+// host reads them there once the stream is idle, without a copy of its own
+static __global__ void __launch_bounds__(RED_NT) reduce_final_kernel(const double* partials, int chunks, const Ctl* ctl,
+                                                                     double* result)
 {
     __shared__ double sh[RED_NT / 32][RED_NV];
     double v[RED_NV] = {0.0, 0.0, 0.0, -INFINITY, INFINITY, 0.0};
@@ -1095,7 +1098,27 @@ static __global__ void __launch_bounds__(RED_NT) reduce_final_kernel(const doubl
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < RED_NV; k++) result[blockIdx.x * RED_NV + k] = v[k];
+        if (blockIdx.x == 0) result[gridDim.x * RED_NV] = (double)ctl->err;
     }
+}
+
+// Rows [row, row + count / nx) of an instance's phi as contiguous doubles for the host (count < 2^31).  note[0] is set when
+// one of them is not finite, note[1] to the error flags of the steps (pinned host memory, as above).
+template <typename P>
+__global__ void __launch_bounds__(256) gather_phi_kernel(const P* phi, const float* lo, int pitch, int nx, unsigned count,
+                                                         const Ctl* ctl, double* out, double* note)
+{
+    const unsigned e = blockIdx.x * 256u + threadIdx.x;
+    bool bad = false;
+    if (e < count) {
+        const unsigned y = e / (unsigned)nx;
+        const long long k = (long long)y * pitch + (e - y * (unsigned)nx);
+        const double p = (double)phi[k] + (lo ? (double)lo[k] : 0.0);
+        out[e] = p;
+        bad = !isfinite(p);
+    }
+    if (__syncthreads_or(bad) && threadIdx.x == 0) note[0] = 1.0;
+    if (e == 0) note[1] = (double)ctl->err;
 }
 
 }  // namespace lbch

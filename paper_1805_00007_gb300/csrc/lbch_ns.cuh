@@ -56,7 +56,7 @@ struct NsArgs {
     C* out;            // of the next one
     C* aux;            // [ny][nb][5][32]: phi, u, mu and p of the current state
     C* phi;            // the handle's padded phi array of the current state
-    C* obs;            // [3][ny nx]: u and p for observation
+    double* obs;       // [3][ny nx]: u and p for observation
     // constants of the form in double with the stencils' 1/12 and 1/6 folded in: kappa/6, a M/6, a/24, K/144, 3 src_f,
     // 3 src_f a/36, 3/tau_f, 3 src/9 and eta/tau_g
     C kappa6, aM6, a24, K144, s3, s3a36, itf3, src9, ieta;
@@ -272,9 +272,9 @@ __global__ void __launch_bounds__(NT) fields_kernel(NsArgs<C> a)
     const C pr = op_mul(C(3) / C(5), op_fma(-C(1.5) * wq<C>(0), op_mul(rho, uu), t));
     if (OBS) {
         const long long N = (long long)a.nx * a.ny, k = (long long)y * a.nx + x;
-        a.obs[k] = ux;
-        a.obs[N + k] = uy;
-        a.obs[2 * N + k] = pr;
+        a.obs[k] = (double)ux;
+        a.obs[N + k] = (double)uy;
+        a.obs[2 * N + k] = (double)pr;
     } else {
         C* w = a.aux + at<AUXS>(a, x, y);
         w[A_PHI] = phi;
