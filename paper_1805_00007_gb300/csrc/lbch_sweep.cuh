@@ -257,8 +257,15 @@ __global__ void __launch_bounds__(SweepShape<S, P, FF, GEN, GEN && (WALLS || !SI
         const bool vb = 2 * lane + 1 >= L::FIRST && 2 * lane + 1 < L::FIRST + L::W && xb >= 0 && xb < I.nx;
         const bool both = va && vb, one = va != vb;
         // whether a node of the strip has ghost images in x (three columns from the domain's edge): the image stores
-        // and their tests are skipped as a whole elsewhere
+        // and their tests are skipped as a whole elsewhere.  A row that has no images in y takes its nodes' one image at
+        // a distance the lane knows (iwa, iwb; GEN: gwa, gwb; 0: none); the other rows, and domains so narrow that a node
+        // may have two images in x, take the general way.  (With the general way on every row of these strips, the SMs
+        // that held them took 99 thousand cycles at 3001 x 1999 where the average took 75.)
         const bool ximg = col0 - GC + L::FIRST < 3 || col0 - GC + L::FIRST + L::W > I.nx - 3;
+        const bool narrow = I.nx < 6;
+        auto image = [&](bool v, int x, int deep) { return !v ? 0 : x < deep ? I.nx : x >= I.nx - deep ? -I.nx : 0; };
+        const int iwa = image(va, xa, 3), iwb = image(vb, xb, 3);
+        [[maybe_unused]] const int gwa = GEN ? image(va, xa, 1) : 0, gwb = GEN ? image(vb, xb, 1) : 0;
         const int wlo = WALLS && I.walls ? 0 : -1000000, whi = WALLS && I.walls ? I.ny - 1 : -1000000;  // wall rows
         const int row0 = I.row0, ylast = I.ny - 3;
         const C* tW = tY1 + 2 * I.ylen;  // Y1, Y2 at the walls y = -1/2, ny - 1/2
@@ -593,6 +600,11 @@ __global__ void __launch_bounds__(SweepShape<S, P, FF, GEN, GEN && (WALLS || !SI
                 *pout = va ? hia : hib;
                 if (FF) *lout = va ? loa : lob;
             }
+            const bool images = yo < 3 || yo >= ylast || (ximg && narrow);  // the general way
+            if (ximg && !images) {
+                if (iwa) pout[iwa] = hia;
+                if (iwb) pout[iwb + (both ? 1 : 0)] = hib;
+            }
             pout += pitch;
             if (FF) lout += pitch;
             if constexpr (GEN) {
@@ -607,13 +619,20 @@ __global__ void __launch_bounds__(SweepShape<S, P, FF, GEN, GEN && (WALLS || !SI
 #pragma unroll
                     for (int q = QOFF; q < 9; q++) gout[(long long)(q - QOFF) * pitch] = to_s<S>(va_[q]);
                 }
+                if (ximg && !images) {
+#pragma unroll
+                    for (int q = QOFF; q < 9; q++) {
+                        if (gwa) gout[(long long)(q - QOFF) * pitch + gwa] = to_s<S>(va_[q]);
+                        if (gwb) gout[(long long)(q - QOFF) * pitch + gwb + (both ? 1 : 0)] = to_s<S>(vb_[q]);
+                    }
+                }
                 gout += NQ * pitch;
-                if (ximg || yo < 3 || yo >= ylast) {
+                if (images) {
                     if (va) store_g_images<S, C, QOFF>(a.g_out, row0, pitch, I.nx, I.ny, I.walls, xa, yo, va_);
                     if (vb) store_g_images<S, C, QOFF>(a.g_out, row0, pitch, I.nx, I.ny, I.walls, xb, yo, vb_);
                 }
             }
-            if (ximg || yo < 3 || yo >= ylast) {
+            if (images) {
                 if (va) store_images(a.phi_out, row0, pitch, I.nx, I.ny, I.walls, xa, yo, hia);
                 if (vb) store_images(a.phi_out, row0, pitch, I.nx, I.ny, I.walls, xb, yo, hib);
             }
