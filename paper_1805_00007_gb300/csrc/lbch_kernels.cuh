@@ -461,6 +461,47 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, in
         : "memory");
 }
 
+// f(xx, yy) for the ghost cells that stand for domain node (x, y): periodic images in x; periodic or (walls) mirror images in
+// y, three deep.  A node has at most one image along each axis unless the domain is narrower than six nodes.  (Straight-line
+// code: a tile on the edge sets the time of a launch of one tile per SM, and as a loop over all images that a node can have
+// these tests were 1 to 5 % of a step on grids of 45 to 1024 squared.)
+template <typename F>
+__device__ __forceinline__ void for_images3(int x, int y, int nx, int ny, int walls, F&& f)
+{
+    const int xa = x < 3 ? x + nx : x >= nx - 3 ? x - nx : x;
+    const int ya = y < 3 ? (walls ? -1 - y : y + ny) : y >= ny - 3 ? (walls ? 2 * ny - 1 - y : y - ny) : y;
+    if (xa != x) f(xa, y);
+    if (ya != y) {
+        f(x, ya);
+        if (xa != x) f(xa, ya);
+    }
+    if (nx >= 6 && ny >= 6) return;
+    const int xb = x < 3 && x >= nx - 3 ? x - nx : x;  // the second image along an axis
+    const int yb = y < 3 && y >= ny - 3 ? (walls ? 2 * ny - 1 - y : y - ny) : y;
+    if (xb != x) {
+        f(xb, y);
+        if (ya != y) f(xb, ya);
+    }
+    if (yb != y) {
+        f(x, yb);
+        if (xa != x) f(xa, yb);
+        if (xb != x) f(xb, yb);
+    }
+}
+
+// The same one deep, for the populations: periodic images in x, and in y unless the instance has walls there.
+template <typename F>
+__device__ __forceinline__ void for_images1(int x, int y, int nx, int ny, int walls, F&& f)
+{
+    const int xa = x == 0 ? nx : x == nx - 1 ? -1 : x;
+    const int ya = walls ? y : y == 0 ? ny : y == ny - 1 ? -1 : y;
+    if (xa != x) f(xa, y);
+    if (ya != y) {
+        f(x, ya);
+        if (xa != x) f(xa, ya);
+    }
+}
+
 // Model III: H(t) of domain node (x, y) and its ghost images one deep (periodic in x; in y unless walls).
 template <typename C>
 __device__ __forceinline__ void store_h(C* H, long long plane, int row0, int pitch, int nx, int ny, int walls, int x,
@@ -566,7 +607,6 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
     constexpr int QOFF = kHalf ? 1 : 0;       // stored plane of population q is q - QOFF
     // at tau_g = 1 the axis populations are staged in a quarter (collide9); not where they round to half
     constexpr bool kQuarter = TAU1 && !kHalf;
-    constexpr int NONE = -0x40000000;
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = smem_aligned128(smem_raw);
@@ -895,30 +935,15 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
             if (edge) {
                 // the node's images in the ghost columns/rows (phi three deep, the populations one deep;
                 // in y only for periodic y, mirror images next to walls)
-                const int xa = gx < 3 ? gx + nx : NONE, xb = gx >= nx - 3 ? gx - nx : NONE;
-                const int ya = gy < 3 ? (walls ? -1 - gy : gy + ny) : NONE;
-                const int yb = gy >= ny - 3 ? (walls ? 2 * ny - 1 - gy : gy - ny) : NONE;
-                for (int iy = 0; iy < 3; iy++) {
-                    const int yy = iy == 0 ? gy : (iy == 1 ? ya : yb);
-                    if (yy == NONE) continue;
-                    for (int ix = 0; ix < 3; ix++) {
-                        const int xx = ix == 0 ? gx : (ix == 1 ? xa : xb);
-                        if (xx == NONE || (ix == 0 && iy == 0)) continue;
-                        a.phi_out[(long long)(I.row0 + yy) * pitch + GC + xx] = hi;
-                    }
-                }
-                const int gxa = gx == 0 ? nx : (gx == nx - 1 ? -1 : NONE);
-                const int gya = walls ? NONE : (gy == 0 ? ny : (gy == ny - 1 ? -1 : NONE));
-                for (int iy = 0; iy < (TAU1 ? 0 : 2); iy++) {
-                    const int yy = iy == 0 ? gy : gya;
-                    if (yy == NONE) continue;
-                    for (int ix = 0; ix < 2; ix++) {
-                        const int xx = ix == 0 ? gx : gxa;
-                        if (xx == NONE || (ix == 0 && iy == 0)) continue;
+                for_images3(gx, gy, nx, ny, walls, [&](int xx, int yy) {
+                    a.phi_out[(long long)(I.row0 + yy) * pitch + GC + xx] = hi;
+                });
+                if (!TAU1)
+                    for_images1(gx, gy, nx, ny, walls, [&](int xx, int yy) {
                         S* oi = a.g_out + ((long long)(I.row0 + yy) * NQ) * pitch + GC + xx;
+#pragma unroll
                         for (int q = QOFF; q < 9; q++) oi[(q - QOFF) * pitch] = to_s<S>(v[q]);
-                    }
-                }
+                    });
             }
         });
         // the stage takes the tile after next once every thread is done with it (the next iteration's

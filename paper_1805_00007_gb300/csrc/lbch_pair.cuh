@@ -360,7 +360,6 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
     constexpr bool kFF = L::FF;
     constexpr bool kShift = sizeof(C) == 4;  // float arithmetic carries g_0 - phi
     constexpr int W6 = L::W6, W3 = L::W3;
-    constexpr int NONE = -0x40000000;
     const Consts<C>& K0 = consts<C>(I);
     const bool model2 = I.model == 2;
 
@@ -382,17 +381,7 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
     // phi(t+2) of a domain node, with its periodic images in the ghost frame (three deep), read by one-step launches
     auto images = [&](int gx, int gy, P hi) {
         if (gx >= 3 && gx < nx - 3 && gy >= 3 && gy < ny - 3) return;
-        const int xa = gx < 3 ? gx + nx : NONE, xb = gx >= nx - 3 ? gx - nx : NONE;
-        const int ya = gy < 3 ? gy + ny : NONE, yb = gy >= ny - 3 ? gy - ny : NONE;
-        for (int iy = 0; iy < 3; iy++) {
-            const int yy = iy == 0 ? gy : (iy == 1 ? ya : yb);
-            if (yy == NONE) continue;
-            for (int ix = 0; ix < 3; ix++) {
-                const int xx = ix == 0 ? gx : (ix == 1 ? xa : xb);
-                if (xx == NONE || (ix == 0 && iy == 0)) continue;
-                phi_out[rb + (long long)yy * pitch + xx] = hi;
-            }
-        }
+        for_images3(gx, gy, nx, ny, 0, [&](int xx, int yy) { phi_out[rb + (long long)yy * pitch + xx] = hi; });
     };
 
     if constexpr (kFF) {

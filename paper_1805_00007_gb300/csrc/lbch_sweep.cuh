@@ -143,19 +143,7 @@ __device__ __forceinline__ void store_images(P* phi_out, long long row0, int pit
                                              int y, P v)
 {
     if (x >= 3 && x < nx - 3 && y >= 3 && y < ny - 3) return;
-    constexpr int NONE = -1000000;
-    const int xa = x < 3 ? x + nx : NONE, xb = x >= nx - 3 ? x - nx : NONE;
-    const int ya = y < 3 ? (walls ? -1 - y : y + ny) : NONE;
-    const int yb = y >= ny - 3 ? (walls ? 2 * ny - 1 - y : y - ny) : NONE;
-    for (int iy = 0; iy < 3; iy++) {
-        const int yy = iy == 0 ? y : (iy == 1 ? ya : yb);
-        if (yy == NONE) continue;
-        for (int ix = 0; ix < 3; ix++) {
-            const int xx = ix == 0 ? x : (ix == 1 ? xa : xb);
-            if (xx == NONE || (ix == 0 && iy == 0)) continue;
-            phi_out[(row0 + yy) * pitch + GC + xx] = v;
-        }
-    }
+    for_images3(x, y, nx, ny, walls, [&](int xx, int yy) { phi_out[(row0 + yy) * pitch + GC + xx] = v; });
 }
 
 // Writes g(t+1) of domain node (x, y) into the ghost cells that stand for it, one deep: periodic images
@@ -164,22 +152,12 @@ template <typename S, typename C, int QOFF>
 __device__ __forceinline__ void store_g_images(S* g_out, long long row0, int pitch, int nx, int ny, int walls, int x, int y,
                                                const C* v)
 {
-    constexpr int NONE = -1000000;
-    const int gxa = x == 0 ? nx : (x == nx - 1 ? -1 : NONE);
-    const int gya = walls ? NONE : (y == 0 ? ny : (y == ny - 1 ? -1 : NONE));
-    if (gxa == NONE && gya == NONE) return;
     constexpr int NQ = 9 - QOFF;
-    for (int iy = 0; iy < 2; iy++) {
-        const int yy = iy == 0 ? y : gya;
-        if (yy == NONE) continue;
-        for (int ix = 0; ix < 2; ix++) {
-            const int xx = ix == 0 ? x : gxa;
-            if (xx == NONE || (ix == 0 && iy == 0)) continue;
-            S* o = g_out + ((row0 + yy) * NQ) * pitch + GC + xx;
+    for_images1(x, y, nx, ny, walls, [&](int xx, int yy) {
+        S* o = g_out + ((row0 + yy) * NQ) * pitch + GC + xx;
 #pragma unroll
-            for (int q = QOFF; q < 9; q++) o[(long long)(q - QOFF) * pitch] = to_s<S>(v[q]);
-        }
-    }
+        for (int q = QOFF; q < 9; q++) o[(long long)(q - QOFF) * pitch] = to_s<S>(v[q]);
+    });
 }
 
 // SINGLE (a handle of one instance): the instance record stays in the launch parameters, and the arithmetic takes
