@@ -174,9 +174,9 @@ lbch_status lb_ch_halo_import(lbch_handle* h, int side, const void* src);
  * step: the library then reads and writes phi only (the stored populations are left unchanged and are
  * not part of the state), with the same results bit for bit.  Until lb_ch_tune chooses otherwise, the
  * kernel is chosen by the size of the handle's grids: LBCH_F32 handles whose instances are all periodic with tau_g = 1
- * and make up to three 32 x 14 tiles per SM (about 200 K nodes) step two steps per launch with the two-step
+ * and make up to two and a half 32 x 14 tiles per SM (about 170 K nodes) step two steps per launch with the two-step
  * kernel; the tile kernel steps LBCH_F64 handles of up to about 900 K nodes and, where some tau_g != 1, float ones of up
- * to about 75 K; the row sweep steps every other handle, and those with a Model III instance. */
+ * to about 100 K; the row sweep steps every other handle, and those with a Model III instance. */
 lbch_status lb_ch_step(lbch_handle* h, long nsteps);
 
 /* Read an observable of instance inst into out (host, sized as lbch_obs states).  Synchronises the
@@ -219,7 +219,8 @@ void* lb_ch_stream(lbch_handle* h);
  * row sweep (warps sweeping strips of 56 or 58 columns, the grid cut into as many as 16, 8, 4 or 12 warps per SM --
  * fewer where its registers allow fewer --; reported as tiles of 56 x 48, 56 x 24, 56 x 12 and 56 x 24 output nodes),
  * the tile kernel (each tile's stencil fields staged in shared memory; 32x16, 32x8 and 16x8 with 256
- * threads and 32x16 with 768 on the float paths; 32x8 and 16x8 with 256 and 32x8 with 512 for LBCH_F64)
+ * threads and 32x16 with 768 on the float paths; 32x8 and 16x8 with 256, 32x8 with 512,
+ * 32x16 with 768 and 32x14 with 704 for LBCH_F64)
  * and, for handles whose instances are all periodic with tau_g = 1 in LBCH_F32 or LBCH_F64, the two-step
  * kernel (two steps per launch from phi on the tile + 6; 32x16, 32x14 and 32x8 with 512 threads and 16x8 with
  * 256 in LBCH_F32; 32x8 with 512, 16x8 with 256, 16x16 with 512 and 32x14 with 1024

@@ -1094,10 +1094,12 @@ void choose_default(lbch_handle* h, int sms)
 {
     if (h->coupled) return;
     const bool tau1 = h->tau1;
-    // the row sweep: on grids so small that sixteen warps per SM would get two rows each or fewer, strips for half as many
-    // warps (eight in double: a quarter) step faster -- 256^2 in float 4.7 against 5.3, double 36 against 54
+    // the row sweep: on grids so small that sixteen warps per SM would get two rows each or fewer (in float at tau_g = 1 five,
+    // a row being shorter there), strips for half as many warps (eight in double: a quarter) step faster: at tau_g = 1 in
+    // float 448^2 4.9 against 5.6, 768^2 7.5 against 7.9, 900^2 8.8 against 8.7; with the populations 384^2 7.5 against
+    // 8.0, 600^2 10.7 against 10.1; double 256^2 36 against 54
     const lbch_handle::SweepCut& cut = h->sw[0][sweep_gen(h)];
-    h->shape = h->prec == LBCH_F64 ? (cut.rows_per <= 8 && !h->model3 ? 2 : 0) : (cut.rows_per <= 2 ? 1 : 0);
+    h->shape = h->prec == LBCH_F64 ? (cut.rows_per <= 8 && !h->model3 ? 2 : 0) : (cut.rows_per <= (h->prec == LBCH_F32 && tau1 ? 5 : 2) ? 1 : 0);
     if (h->model3) return;
     auto tiles = [&](int k) { return h->ps[k].total_tiles; };
     if (h->prec == LBCH_F64) {
@@ -1113,16 +1115,18 @@ void choose_default(lbch_handle* h, int sms)
     }
     if (h->prec == LBCH_F16S && tau1) return;  // the tile kernel would round the populations to half
     if (!tau1) {
-        // with the populations: small tiles on small grids (100^2: 3.0 against the sweep's 3.6; 160^2: 3.5), one wave of
-        // 32 x 16 (256^2: 4.6 against 5.8), then the row sweep (360^2: 7.1 against 7.4)
-        if (2 * tiles(2) <= 3 * sms) { h->force_tile = true; h->shape = 2; }
+        // with the populations: small tiles on small grids (100^2: 2.9 against the sweep's 4.5; 200^2: 4.1), one wave of
+        // 32 x 16 (256^2: 4.5 against 6.0), 32 x 8 up to three per SM (300^2: 5.7 against 6.1), then the row sweep
+        // (384^2: 7.5 against 7.9)
+        if (2 * tiles(2) <= 5 * sms) { h->force_tile = true; h->shape = 2; }
         else if (tiles(3) <= sms) { h->force_tile = true; h->shape = 3; }
+        else if (tiles(1) <= 3 * sms) { h->force_tile = true; h->shape = 1; }
         return;
     }
-    // tau_g = 1 in float: the two-step kernel on periodic grids up to three of its 32 x 14 tiles per SM -- 16 x 8 and 32 x 8
-    // tiles while every SM gets one (100^2: 1.6 per step against the row sweep's 4.0; 160^2: 1.8), 32 x 14 up to two
-    // (256^2: 2.1 against 4.7; 300^2: 3.1), 32 x 16 up to two (360^2: 3.6 against 5.5), 32 x 14 up to three (400^2: 4.7
-    // against 5.6) --, otherwise the row sweep (512^2: 6.2).  The odd last step of a call, and taped steps, take
+    // tau_g = 1 in float: the two-step kernel on periodic grids up to two and a half of its 32 x 14 tiles per SM -- 16 x 8
+    // and 32 x 8 tiles while every SM gets one (100^2: 1.5 per step against the row sweep's 3.7; 160^2: 1.8), 32 x 14 up to
+    // two (256^2: 2.0 against 4.3; 320^2: 3.1 against 4.4), 32 x 16 up to two (384^2: 3.6 against 5.1), 32 x 14 from there
+    // (400^2: 4.7 against 5.0) --, otherwise the row sweep (448^2: 4.9 against 5.9).  The odd last step of a call, and taped steps, take
     // the one-step kernel that is faster there: 16 x 8 tiles up to three per SM (100^2: 2.7 against 4.0).
     if (!pair_ok(h)) return;
     auto pairs = [&](int k) { return h->pr[k].total_tiles; };
@@ -1131,7 +1135,7 @@ void choose_default(lbch_handle* h, int sms)
     else if (pairs(3) <= sms) h->pshape = 3;
     else if (pairs(1) <= 2 * sms) h->pshape = 1;
     else if (pairs(0) <= 2 * sms) h->pshape = 0;
-    else if (pairs(1) <= 3 * sms) h->pshape = 1;
+    else if (2 * pairs(1) <= 5 * sms) h->pshape = 1;
     else h->pair = false;
     if (h->pair && tiles(2) <= 3 * sms) { h->force_tile = true; h->shape = 2; }
 }
