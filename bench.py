@@ -33,12 +33,12 @@ from paper_1805_00007_gb300 import workloads as wl  # noqa: E402
 REV_N = 256
 METRIC = "MLUPS and % HBM roofline (FP32 vs FP64 step) at stated phi error vs FP64 oracle"
 
-# FP32 operations per lattice update of the row-sweep step at tau_g = 1, Model II, float-float phi: the
-# operations of the per-node helpers (a fused multiply-add counts 2): mu 23, D = div(phi u) 34, grad mu and
-# grad D 28, force 11, velocity 4, equilibrium + source + collision 55, streaming sum and TwoSum 14.
-FLOPS_PER_LU_TAU1 = 169
+# FP32 operations per lattice update of the row-sweep step at tau_g = 1, Model II, float-float phi, the stencils taken
+# column first and the constants folded (a fused multiply-add counts 2): 34 additions, 17 products and 30 fused
+# multiply-adds per node, from the instruction counts of a launch on 3001 x 1999 over the nodes it forms, halo included.
+FLOPS_PER_LU_TAU1 = 111
 # The FP64 step does the same operations without the TwoSum (6 fewer) and with a reciprocal refined by two
-# Newton steps (6 more): 169 as well.
+# Newton steps (6 more): 111 as well.
 SMS, FP32_LANES_PER_SM, FP64_LANES_PER_SM = 152, 128, 2
 
 # Algorithmic HBM bytes per lattice update of the general step (any tau_g): the nine populations read and

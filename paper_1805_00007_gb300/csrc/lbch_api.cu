@@ -4,7 +4,7 @@
 // the instance table, the separable velocity tables, the TMA tensor maps, the step counter and the
 // reduction scratch.  It derives the model constants from the parameters (Eqs. betakappa, rho, F2-1,
 // the mobility relation after Eq. phit3 and the Peclet number of Sec. III.A), launches the persistent
-// step kernel -- replayed from CUDA graphs of 64 steps -- and the reductions behind lb_ch_observe.
+// step kernels -- replayed from CUDA graphs of 64 and 512 steps -- and the reductions behind lb_ch_observe.
 #include "lbch.h"
 #include "lbch_adjoint.cuh"
 #include "lbch_internal.h"

@@ -1,7 +1,8 @@
 // lbch_kernels.cuh -- sm_103a device code of the Cahn-Hilliard lattice Boltzmann step.
 //
 // Method: Zhang, Guo & Liang, arXiv:1805.00007, Sec. II (Eqs. LB, geq, liangFi, macroscopicg, mu, bulk,
-// betakappa, rho, t0-phiu, mark3).  The step is one fused, memory-bound kernel; no tensor cores.
+// betakappa, rho, t0-phiu, mark3).  The step is one fused kernel; no tensor cores (a stencil has no contraction).  This file
+// holds the arithmetic that every form of the step shares, and the tile kernel.
 //
 // Storage ("padded image layout").  Every stored row has the same pitch.  An instance occupies
 // ny + 2*GR consecutive stored rows; domain node (x, y) sits at stored row row0 + y, column GC + x.  The
@@ -14,10 +15,10 @@
 // Per step a persistent CTA walks its tiles (TX x TY output nodes) with a two-stage TMA pipeline:
 // while tile k is computed, the population box (tile + 1 halo) and the phi box (tile + 3 halo) of the
 // next tile are in flight.  For each tile the CTA
-//   1. forms phi and the flux phi u on tile + 3 (velocity from per-instance separable tables),
-//   2. computes mu = f'(phi) - kappa lap phi and D = div(phi u) on tile + 2,
-//   3. on tile + 1 computes grad mu, grad D, the force F, g_eq and S and collides, in place in the box,
-//   4. pulls g*_i(x - c_i) from shared memory for every tile node (halfway bounce-back at walls) and
+//   1. computes mu = f'(phi) - kappa lap phi and D = div(phi u) on tile + 2 (velocity from per-instance separable tables;
+//      stencils column first, in double through column sums in shared memory),
+//   2. on tile + 1 computes grad mu, grad D, the force F, g_eq and S and collides, in place in the box,
+//   3. pulls g*_i(x - c_i) from shared memory for every tile node (halfway bounce-back at walls) and
 //      stores g(t+1) and phi(t+1), with the ghost images the next step's boxes need.
 // HBM traffic per lattice update is one read and one write of the stored populations and of phi; the
 // overlap of neighbouring tiles' boxes is served from L2.
