@@ -598,10 +598,15 @@ __global__ void __launch_bounds__(SweepShape<S, P, FF, GEN, GEN && (WALLS || !SI
                     for (int q = QOFF; q < 9; q++) gout[(long long)(q - QOFF) * pitch] = to_s<S>(va_[q]);
                 }
                 if (ximg && !images) {
+                    if (gwa) {
+                        S* o = gout + gwa;
 #pragma unroll
-                    for (int q = QOFF; q < 9; q++) {
-                        if (gwa) gout[(long long)(q - QOFF) * pitch + gwa] = to_s<S>(va_[q]);
-                        if (gwb) gout[(long long)(q - QOFF) * pitch + gwb + (both ? 1 : 0)] = to_s<S>(vb_[q]);
+                        for (int q = QOFF; q < 9; q++) o[(long long)(q - QOFF) * pitch] = to_s<S>(va_[q]);
+                    }
+                    if (gwb) {
+                        S* o = gout + gwb + (both ? 1 : 0);
+#pragma unroll
+                        for (int q = QOFF; q < 9; q++) o[(long long)(q - QOFF) * pitch] = to_s<S>(vb_[q]);
                     }
                 }
                 gout += NQ * pitch;
