@@ -485,8 +485,19 @@ lbch_status check_params(const lbch_params& p, int k)
     return LBCH_OK;
 }
 
+// The force divides by v = ra phi + rb = -(144/src) rho (lbch_kernels.cuh), whose magnitude must stay a normal number with a
+// normal reciprocal (node_rcp).  Below, the exponent that v has room for, with 2^26 and more in hand for phi beyond its
+// bulk values, and the most by which the unit of the chemical potential is changed to get there.
+constexpr int kForceExp(int prec) { return prec == LBCH_F64 ? 960 : 100; }
+constexpr int kUnitShift = 80;
+
 // Derived constants of the model for one instance.
-void derive(const lbch_params& p, InstDev& d)
+//
+// phi depends on the unit of mu, sigma and the densities only through ratios: with mu, beta, kappa, rho divided by 2^k and eta
+// multiplied by it every step is the same, bit for bit (a power of two rounds nothing).  Densities so large that v would
+// leave its range (in float at tau_g = 1 its reciprocal does at rho = 3e35 and rb at 1.2e36) are taken in such a unit;
+// k = 0 for all others.  Where even that leaves v too large, the force is below any effect and v is held at the limit.
+void derive(const lbch_params& p, int prec, InstDev& d)
 {
     const double cs2 = 1.0 / 3.0;
     const double dphi = std::fabs(p.phiA - p.phiB);
@@ -503,6 +514,14 @@ void derive(const lbch_params& p, InstDev& d)
     c.omt = 1.0 - 1.0 / p.tau;
     c.src = 1.0 - 1.0 / (2.0 * p.tau);
     c.phiA = p.phiA; c.phiB = p.phiB;
+    const double rho = std::max(std::fabs(c.a) * std::max(std::fabs(p.phiA), std::fabs(p.phiB)), std::fabs(c.b));
+    const int over = rho > 0.0 && std::isfinite(rho) ? std::ilogb(rho) + std::ilogb(144.0 / c.src) + 2 - kForceExp(prec) : 0;
+    if (over > 0 && p.vel != LBCH_VEL_COUPLED) {  // (the coupled flow does not use v, and its pressure has the user's unit)
+        const int k = std::min(over, kUnitShift);
+        c.beta = std::ldexp(c.beta, -k); c.kappa = std::ldexp(c.kappa, -k);
+        c.a = std::ldexp(c.a, -k); c.b = std::ldexp(c.b, -k);
+        c.eta = std::ldexp(c.eta, k);
+    }
     c.cF1 = 2.0 * p.tau - 1.0 + 3.0 * c.K;                               // Eq. F2-1: coefficient of d_t F1
     c.cmu = 3.0 * cs2 * c.eta * c.K;                                     // and of d_t grad mu
     Consts<float>& f = d.cf;
@@ -512,8 +531,12 @@ void derive(const lbch_params& p, InstDev& d)
     f.cF1 = (float)c.cF1; f.cmu = (float)c.cmu;
     // the products the per-node arithmetic takes (lbch_kernels.cuh), formed in double and rounded once
     const double k3 = c.src / 12.0;  // 3 w_5 src
-    const double k[9] = {4.0 * c.beta, -2.0 * c.beta * (p.phiA + p.phiB), c.itau / 36.0 * c.eta,
-                         -144.0 * c.a / c.src, -144.0 * c.b / c.src, k3 * c.K / 12.0, k3, c.cF1 / k3, c.cmu / 12.0};
+    double k[9] = {4.0 * c.beta, -2.0 * c.beta * (p.phiA + p.phiB), c.itau / 36.0 * c.eta,
+                   -144.0 * c.a / c.src, -144.0 * c.b / c.src, k3 * c.K / 12.0, k3, c.cF1 / k3, c.cmu / 12.0};
+    if (over > kUnitShift) {
+        k[3] = 0.0;
+        k[4] = -std::ldexp(1.0, kForceExp(prec));
+    }
     auto products = [&](auto& o) {
         using T = std::remove_reference_t<decltype(o.beta)>;
         o.b4 = (T)k[0]; o.b2s = (T)k[1]; o.kM = (T)k[2]; o.ra = (T)k[3]; o.rb = (T)k[4];
@@ -1187,7 +1210,7 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
         const lbch_params& p = params[k];
         InstDev& d = h->inst[k];
         std::memset(&d, 0, sizeof d);
-        derive(p, d);
+        derive(p, prec, d);
         d.nx = p.nx;
         d.ny = p.ny;
         d.slab = slab ? 1 : 0;
