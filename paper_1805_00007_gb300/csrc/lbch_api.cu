@@ -445,8 +445,7 @@ cudaError_t launch_step(lbch_handle* h, int parity)
 cudaError_t time_table(lbch_handle* h, int steps)
 {
     if (!h->timed) return cudaSuccess;
-    const int n = steps * h->n_inst;
-    time_table_kernel<<<(n + 127) / 128, 128, 0, h->stream>>>(h->d_inst, h->n_inst, h->ctl, steps, h->d_T);
+    time_table_kernel<<<time_table_blocks(steps, h->n_inst), TIME_NT, 0, h->stream>>>(h->d_inst, h->n_inst, h->ctl, steps, h->d_T);
     return cudaGetLastError();
 }
 
