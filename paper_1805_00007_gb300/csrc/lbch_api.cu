@@ -871,20 +871,25 @@ lbch_status run_reduce(lbch_handle* h)
 }
 
 // Instance inst's phi to `out`: made doubles on the device, in the buffer of the next state (which the next step fills
-// completely), as many rows at a time as it holds, and copied from there to the caller's memory.  (256 x 1024 in double: 49
-// us, against 338 as a copy to pinned memory, a second one and a search for non-finite values on the host; 1024 x 1024 in
-// float: 107 against 1337.)
+// completely), as many rows at a time as it holds (a float state's takes two turns), and copied from there to the caller's
+// memory.  (256 x 1024 in double: 49 us, against 338 as a copy to pinned memory, a second one and a search for non-finite
+// values on the host; 1024 x 1024 in float: 107 against 1337.)  Of small fields the copies' own calls are most of the time:
+// up to 2^13 nodes of a double state and 2^15 of a float one the kernel stores into the pinned staging buffer, and the host
+// copies from there (us, copied -> staged: double 16^2 22 -> 16, 80^2 22 -> 20, 128^2 22 -> 26; float 32^2 37 -> 16,
+// 100^2 37 -> 20, 160^2 38 -> 28, 224^2 38 -> 40).
 lbch_status read_phi(lbch_handle* h, int inst, double* out)
 {
     const InstDev& d = h->inst[inst];
     const int parity = cur_buf(h);
-    lbch_status s = stage(h, 2 * sizeof(double));
+    const size_t nodes = (size_t)d.nx * d.ny;
+    const bool staged = nodes <= (h->phi_elem == 8 ? 1u << 13 : 1u << 15);
+    lbch_status s = stage(h, (2 + (staged ? nodes : 0)) * sizeof(double));
     if (s != LBCH_OK) return s;
     double* note = h->h_stage;
     note[0] = note[1] = 0.0;
-    const size_t cells = (size_t)h->rows * h->pitch * h->phi_elem / sizeof(double);
+    const size_t cells = staged ? nodes : (size_t)h->rows * h->pitch * h->phi_elem / sizeof(double);
     const long long fit = (long long)std::min<size_t>(cells, 1u << 30) / d.nx;  // rows, at least one: pitch > nx, two rows or more
-    double* buf = static_cast<double*>(h->phi[parity ^ 1]);
+    double* buf = staged ? note + 2 : static_cast<double*>(h->phi[parity ^ 1]);
     cudaError_t e = cudaSuccess;
     for (long long y = 0; y < d.ny && e == cudaSuccess; y += fit) {
         const unsigned count = (unsigned)(std::min<long long>(fit, d.ny - y) * d.nx);
@@ -897,11 +902,12 @@ lbch_status read_phi(lbch_handle* h, int inst, double* out)
             gather_phi_kernel<float><<<nb, 256, 0, h->stream>>>((const float*)h->phi[parity] + off, h->lo[parity] ? h->lo[parity] + off : nullptr,
                                                                 h->pitch, d.nx, count, h->ctl, buf, note);
         e = cudaGetLastError();
-        if (e == cudaSuccess)
+        if (e == cudaSuccess && !staged)
             e = cudaMemcpyAsync(out + (size_t)y * d.nx, buf, (size_t)count * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
     }
     s = finish_read(h, e, note + 1);
     if (s != LBCH_OK) return s;
+    if (staged) std::memcpy(out, buf, nodes * sizeof(double));
     return note[0] == 0.0 ? LBCH_OK : fail(LBCH_ENONFINITE, "phi holds non-finite values");
 }
 
