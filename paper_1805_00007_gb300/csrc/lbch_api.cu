@@ -281,18 +281,20 @@ cudaError_t prepare_sweep(lbch_handle* h, bool gen, SweepFit* fit)
     }
 }
 
-// Rows per strip of the row sweep, for strips of `width` columns over the handle's instances shared out among `warps`
-// resident warps: the length that takes the fewest row steps, a strip of R rows taking R + 6 of them and the strips
-// coming in rounds of `warps` (one round, where the grid allows strips that long).
-int sweep_rows(const lbch_handle* h, const SweepFit& fit, int warps)
+// The strips side by side on the handle's instances, by the number of their rows.
+using StripsByRows = std::map<int, long long>;
+
+// Rows per strip of the row sweep, the strips shared out among `warps` resident warps: the length that takes the fewest row
+// steps, a strip of R rows taking R + 6 of them and the strips coming in rounds of `warps` (one round, where the grid
+// allows strips that long).
+int sweep_rows(const StripsByRows& strips, int warps)
 {
-    int most = 1, best = 1;
-    for (const InstDev& d : h->inst) most = std::max(most, d.ny);
+    const int most = strips.rbegin()->first;
+    int best = 1;
     long long best_cost = -1;
     for (int R = 1; R <= most; R += std::max(1, R / 32)) {
         long long items = 0;
-        for (const InstDev& d : h->inst)
-            items += (long long)((d.nx + fit.lead + fit.width - 1) / fit.width) * ((d.ny + R - 1) / R);
+        for (const auto& s : strips) items += s.second * ((s.first + R - 1) / R);
         const long long cost = (items + warps - 1) / warps * (R + 6);
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
@@ -301,10 +303,6 @@ int sweep_rows(const lbch_handle* h, const SweepFit& fit, int warps)
     }
     return best;
 }
-
-// Cut the handle's grids into the strips of configuration k (gen: of the form with the populations), side by side and
-// row block after row block of one instance after the other, so that neighbouring strips go to one block's warps.
-cudaError_t cut_sweep(lbch_handle* h, int k, bool gen, const SweepFit& fit);
 
 // Dynamic shared memory of the step kernel, and the persistent grid that fits the device, for shape k.
 template <typename C, typename S, typename P, int TX, int TY, int NTT = NT>
@@ -733,10 +731,12 @@ int sweep_block(const SweepFit& fit, long long n)
     return nw;
 }
 
-cudaError_t cut_sweep(lbch_handle* h, int k, bool gen, const SweepFit& fit)
+// Cut the handle's grids into the strips of configuration k (gen: of the form with the populations), side by side and
+// row block after row block of one instance after the other, so that neighbouring strips go to one block's warps.
+cudaError_t cut_sweep(lbch_handle* h, int k, bool gen, const SweepFit& fit, const StripsByRows& by_rows)
 {
     lbch_handle::SweepCut& sc = h->sw[k][gen];
-    const int R = sweep_rows(h, fit, std::min(kSweepWarps[k], fit.warps) * fit.sms);
+    const int R = sweep_rows(by_rows, std::min(kSweepWarps[k], fit.warps) * fit.sms);
     std::vector<SweepItem> items;
     sc.rows_per = 0;
     for (int i = 0; i < h->n_inst; i++) {
@@ -758,6 +758,19 @@ cudaError_t cut_sweep(lbch_handle* h, int k, bool gen, const SweepFit& fit)
     cudaError_t e = dalloc(h, &sc.d_items, sizeof(SweepItem) * items.size());
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(sc.d_items, items.data(), sizeof(SweepItem) * items.size(), cudaMemcpyHostToDevice, h->stream);
+    return e;
+}
+
+// ... of every configuration of the form.  A handle with tau_g = 1 everywhere steps without the populations, and cuts for
+// the other form when the test hook asks for it.
+cudaError_t cut_sweeps(lbch_handle* h, bool gen)
+{
+    SweepFit fit;
+    cudaError_t e = prepare_sweep(h, gen, &fit);
+    if (e != cudaSuccess) return e;
+    StripsByRows by_rows;  // (instance by instance for every length tried, the cuts of 20 000 instances took 14 ms)
+    for (const InstDev& d : h->inst) by_rows[d.ny] += (d.nx + fit.lead + fit.width - 1) / fit.width;
+    for (int sk = 0; sk < kSweepShapes && e == cudaSuccess; sk++) e = cut_sweep(h, sk, gen, fit, by_rows);
     return e;
 }
 
@@ -1286,11 +1299,7 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     int sms = 0;
     CKI(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     if (!coupled) {
-        for (int gen = h->tau1 ? 0 : 1; gen < 2; gen++) {  // (with tau_g = 1 the populations are kept for tests only)
-            SweepFit fit;
-            CKI(prepare_sweep(h, gen, &fit));
-            for (int sk = 0; sk < kSweepShapes; sk++) CKI(cut_sweep(h, sk, gen, fit));
-        }
+        CKI(cut_sweeps(h, !h->tau1));
         for (int sk = 0; sk < kPairShapes && prec != LBCH_F16S; sk++) {
             CKI(lbch_prepare_pair(h, sk));
             CKI(dalloc(h, &h->pr[sk].d_tile_begin, sizeof(int) * (n_inst + 1)));
@@ -2003,6 +2012,7 @@ lbch_status lb_ch_test_hook(lbch_handle* h, int hook, long value)
         return LBCH_OK;
     }
     if (hook == LBCH_HOOK_GENERAL_PATH) {
+        if (value && h->tau1 && h->sw[0][1].n_items == 0) CK(cut_sweeps(h, true));
         h->force_general = value != 0;
         drop_graphs(h);
         return LBCH_OK;
