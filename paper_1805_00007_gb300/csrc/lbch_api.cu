@@ -1305,43 +1305,7 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
             CKI(dalloc(h, &h->pr[sk].d_tile_begin, sizeof(int) * (n_inst + 1)));
             CKI(cudaMemcpyAsync(h->pr[sk].d_tile_begin, pair_begin[sk].data(), sizeof(int) * (n_inst + 1),
                                 cudaMemcpyHostToDevice, h->stream));
-            // each tile's velocity tables over the tile + 6 (periodically wrapped), contiguous per tile so that
-            // one bulk copy brings them (the layout of PairShape: X1, X2 by column, Y1, Y2 by row, 16-byte
-            // padded)
-            const Shape sh = pair_shape(prec, sk);
-            const int W6 = sh.tx + 12, H6 = sh.ty + 12;
-            const size_t esz = prec == LBCH_F64 ? 8 : 4;
-            const size_t stride = ((size_t)(2 * (W6 + H6)) * esz + 15) / 16 * 16 / esz;
-            std::vector<double> tt((size_t)h->pr[sk].total_tiles * stride, 0.0);
-            for (int k = 0; k < n_inst; k++) {
-                const InstDev& d = h->inst[k];
-                const double* X1 = &tabs[d.tab];
-                const double* X2 = X1 + h->pitch;
-                const double* Y1 = X2 + h->pitch;
-                const double* Y2 = Y1 + d.ylen;
-                const int tiles_x = (d.nx + sh.tx - 1) / sh.tx, tiles_y = (d.ny + sh.ty - 1) / sh.ty;
-                for (int l = 0; l < tiles_x * tiles_y; l++) {
-                    const int x0 = (l % tiles_x) * sh.tx, y0 = (l / tiles_x) * sh.ty;
-                    double* o = &tt[(size_t)(pair_begin[sk][k] + l) * stride];
-                    for (int c = 0; c < W6; c++) {
-                        const int x = ((x0 - 6 + c) % d.nx + d.nx) % d.nx;
-                        o[c] = X1[GC + x];
-                        o[W6 + c] = X2[GC + x];
-                    }
-                    for (int r = 0; r < H6; r++) {
-                        const int y = ((y0 - 6 + r) % d.ny + d.ny) % d.ny;
-                        o[2 * W6 + r] = Y1[GR + y];
-                        o[2 * W6 + H6 + r] = Y2[GR + y];
-                    }
-                }
-            }
-            CKI(dalloc(h, &h->pr[sk].d_ttabs, tt.size() * esz));
-            if (prec == LBCH_F64) {
-                CKI(cudaMemcpyAsync(h->pr[sk].d_ttabs, tt.data(), tt.size() * esz, cudaMemcpyHostToDevice, h->stream));
-            } else {
-                std::vector<float> tf(tt.begin(), tt.end());  // rounded as the float tables are
-                CKI(cudaMemcpyAsync(h->pr[sk].d_ttabs, tf.data(), tf.size() * esz, cudaMemcpyHostToDevice, h->stream));
-            }
+            CKI(dalloc(h, &h->pr[sk].d_ttabs, lbch_pair_tables_bytes(h, sk)));
         }
     }
     const size_t cells = (size_t)h->rows * h->pitch;
@@ -1398,6 +1362,7 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     CKI(cudaMemcpyAsync(h->d_node_begin, h->node_begin.data(), sizeof(long long) * (n_inst + 1), cudaMemcpyHostToDevice, h->stream));
     CKI(cudaMemcpyAsync(h->d_tabs, tabs.data(), sizeof(double) * tabs.size(), cudaMemcpyHostToDevice, h->stream));
     CKI(cudaMemcpyAsync(h->d_tabs_f, tabs_f.data(), sizeof(float) * tabs_f.size(), cudaMemcpyHostToDevice, h->stream));
+    for (int sk = 0; sk < kPairShapes && h->pr[sk].d_ttabs; sk++) CKI(lbch_pair_tables(h, sk));
     CKI(cudaMemsetAsync(h->ctl, 0, sizeof(Ctl), h->stream));
     for (int k = 0; k < 2; k++) {
         CKI(cudaMemsetAsync(h->g[k], 0, gbytes, h->stream));

@@ -154,6 +154,9 @@ LBCH_INTERNAL cudaError_t lbch_prepare_sweep_f16s_m3(lbch_handle* h, bool gen, S
 // Two-step launches and set-up (lbch_pair.cu); pshape names a pair_shape().
 LBCH_INTERNAL cudaError_t lbch_launch_pair(lbch_handle* h, int parity);
 LBCH_INTERNAL cudaError_t lbch_prepare_pair(lbch_handle* h, int k);
+// Shape k's velocity tables, every tile's own: their bytes, and the launch that forms them from the handle's.
+LBCH_INTERNAL size_t lbch_pair_tables_bytes(const lbch_handle* h, int k);
+LBCH_INTERNAL cudaError_t lbch_pair_tables(lbch_handle* h, int k);
 // Launch limits of a kernel on a device, set and queried once per process (they depend on nothing else) and
 // served from a table afterwards, so that making a handle does not repeat them for every kernel it may run:
 // lbch_kernel_smem lets `kern` use `smem` bytes of dynamic shared memory; lbch_kernel_fit gives how many CTAs

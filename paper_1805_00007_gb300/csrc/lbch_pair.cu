@@ -15,7 +15,6 @@ cudaError_t launch_pair_v(lbch_handle* h, int parity)
     a.inst = h->d_inst;
     a.tile_begin = ps.d_tile_begin;
     a.ttabs = static_cast<const C*>(ps.d_ttabs);
-    static_assert(L::TAB_STRIDE * sizeof(C) == L::TAB_BYTES, "the host lays the tables out with this stride");
     a.n_inst = h->n_inst;
     a.total_tiles = ps.total_tiles;
     a.pitch = h->pitch;
@@ -61,8 +60,57 @@ cudaError_t prepare_pair_v(lbch_handle* h, int k)
     return cudaSuccess;
 }
 
+// Every tile's velocity tables over the tile + 6, periodically wrapped, contiguous per tile so that one bulk copy brings
+// them: X1, X2 by column, Y1, Y2 by row, padded to 16 bytes.  One value per thread, once per handle.  (Formed on the host and copied, the
+// four shapes' tables took 4.3 of the 9.1 ms in which a 1024^2 float handle is set up.)
+template <typename C>
+__global__ void __launch_bounds__(256) pair_tables_kernel(const InstDev* inst, int n_inst, const int* tile_begin, const C* tabs,
+                                                          int pitch, int tx, int ty, int stride, long long count, C* out)
+{
+    const long long e = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (e >= count) return;
+    const int t = (int)(e / stride), i = (int)(e - (long long)t * stride);
+    const int k = find_inst(tile_begin, n_inst, t), local = t - tile_begin[k];
+    const InstDev& I = inst[k];
+    const int tiles_x = (I.nx + tx - 1) / tx, w6 = tx + 12, h6 = ty + 12;
+    const C* X = tabs + I.tab;
+    const C* Y = X + 2 * pitch;
+    C v = C(0);
+    if (i < 2 * w6) {
+        const int q = i >= w6;
+        v = X[q * pitch + GC + wrap(local % tiles_x * tx - 6 + i - q * w6, I.nx)];
+    } else if (i < 2 * w6 + 2 * h6) {
+        const int j = i - 2 * w6, q = j >= h6;
+        v = Y[q * I.ylen + GR + wrap(local / tiles_x * ty - 6 + j - q * h6, I.ny)];
+    }
+    out[e] = v;
+}
+
+template <typename C> cudaError_t pair_tables_t(lbch_handle* h, int k)
+{
+    const Shape sh = pair_shape(h->prec, k);
+    const int stride = pair_table_stride<C>(sh.tx, sh.ty);
+    const long long count = (long long)h->pr[k].total_tiles * stride;
+    pair_tables_kernel<C><<<(unsigned)((count + 255) / 256), 256, 0, h->stream>>>(
+        h->d_inst, h->n_inst, h->pr[k].d_tile_begin, tables<C>(h), h->pitch, sh.tx, sh.ty, stride, count,
+        static_cast<C*>(h->pr[k].d_ttabs));
+    return cudaGetLastError();
+}
+
 }  // namespace
 }  // namespace lbch
+
+size_t lbch_pair_tables_bytes(const lbch_handle* h, int k)
+{
+    const Shape sh = pair_shape(h->prec, k);
+    return h->prec == LBCH_F64 ? (size_t)h->pr[k].total_tiles * lbch::pair_table_stride<double>(sh.tx, sh.ty) * 8
+                               : (size_t)h->pr[k].total_tiles * lbch::pair_table_stride<float>(sh.tx, sh.ty) * 4;
+}
+
+cudaError_t lbch_pair_tables(lbch_handle* h, int k)
+{
+    return h->prec == LBCH_F64 ? lbch::pair_tables_t<double>(h, k) : lbch::pair_tables_t<float>(h, k);
+}
 
 // The shapes are those of pair_shape() (lbch_internal.h), in its order.
 cudaError_t lbch_launch_pair(lbch_handle* h, int parity)

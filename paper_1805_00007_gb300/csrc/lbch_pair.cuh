@@ -41,6 +41,12 @@ struct PairArgs {
     int debug_skip;         // test hook: CTA 0 never issues its first table copy (its bounded wait runs out)
 };
 
+// Values of a tile's velocity tables: X1, X2 over the TX + 12 columns, Y1, Y2 over the TY + 12 rows, padded to 16 bytes
+template <typename C> __host__ __device__ constexpr int pair_table_stride(int tx, int ty)
+{
+    return (int)((2 * (tx + ty + 24) * sizeof(C) + 15) / 16 * 16 / sizeof(C));
+}
+
 // Shared-memory regions, each centred on the tile: region k spans the tile plus k nodes on every side.
 template <typename C, typename P, int TX, int TY>
 struct PairShape {
@@ -59,10 +65,8 @@ struct PairShape {
     static constexpr size_t OFF_D = OFF_MU + a128(N5 * sizeof(C));
     static constexpr size_t OFF_POST = OFF_D + a128(N5 * sizeof(C));
     static constexpr size_t OFF_TAB = OFF_POST + a128(9 * N4 * sizeof(C));
-    // a tile's velocity tables: X1, X2 over the W6 columns, Y1, Y2 over the H6 rows, padded to 16 bytes
-    static constexpr int TAB_N = 2 * W6 + 2 * H6;
-    static constexpr unsigned TAB_BYTES = (TAB_N * sizeof(C) + 15) / 16 * 16;
-    static constexpr int TAB_STRIDE = TAB_BYTES / sizeof(C);
+    static constexpr int TAB_STRIDE = pair_table_stride<C>(TX, TY);  // a tile's velocity tables
+    static constexpr unsigned TAB_BYTES = TAB_STRIDE * sizeof(C);
     // the Y tables times the two steps' time factors (time-dependent flows): Y1, Y2 for step t, then for t + 1
     static constexpr size_t OFF_YT = OFF_TAB + a128(TAB_BYTES);
     static constexpr size_t BYTES = OFF_YT + a128(4 * H6 * sizeof(C)) + 128;  // + alignment slack
