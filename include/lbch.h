@@ -273,8 +273,8 @@ lbch_status lb_ch_step_taped(lbch_handle* h, long nsteps, void* tape);
 lbch_status lb_ch_adjoint_sweep(lbch_handle* h, const void* tape, long n0, long nsteps);
 
 /* Test hook for the failure path of the step kernel's bounded waits.  With hook
- * LBCH_HOOK_SKIP_FIRST_LOAD and value != 0, the next step launches run without CUDA graphs, on the tile kernel
- * where the handle would step with the row sweep (which has no such wait), and their
+ * LBCH_HOOK_SKIP_FIRST_LOAD and value != 0, the next step launches run without CUDA graphs, a handle that
+ * steps with the row sweep (which has no such wait) goes over to the tile kernel and its first shape, and the launches'
  * first thread block never issues its first tile copy, so its bounded wait runs out (after about a
  * second); the kernel then returns cleanly and the next lb_ch_observe reports LBCH_ETIMEOUT.  The
  * handle's state is not advanced correctly afterwards and should be freed.  With hook

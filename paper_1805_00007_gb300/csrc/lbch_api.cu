@@ -216,13 +216,12 @@ cudaError_t launch_step_t(lbch_handle* h, int parity)
 }
 
 // The row-sweep kernel steps the handle (its shape index then names a sweep configuration), without the
-// populations when every instance has tau_g = 1; the tile kernel only when a test asks for it.  When the
+// populations when every instance has tau_g = 1; the tile kernel where force_tile says so (choose_default, lb_ch_tune).  When the
 // two-step kernel is selected (and applies), it takes the steps two at a time and the one-step kernel
 // takes an odd last step.
 inline bool use_pair(const lbch_handle* h) { return h->pair && pair_ok(h); }
-// (the sweep has no bounded wait to run out: with the test hook that withholds a copy, the tile kernel steps instead)
-inline bool use_sweep(const lbch_handle* h) { return !h->force_tile && !h->coupled && !h->debug_skip; }
-// sweep configurations built for the handle (those with Model III: the two unrolled ones)
+inline bool use_sweep(const lbch_handle* h) { return !h->force_tile && !h->coupled; }
+// sweep configurations of the handle's list
 inline int n_sweep_shapes(const lbch_handle* h) { return h->model3 ? kM3SweepShapes : kSweepShapes; }
 inline int n_active(const lbch_handle* h)
 {
@@ -1953,6 +1952,11 @@ lbch_status lb_ch_test_hook(lbch_handle* h, int hook, long value)
     if (!h) return fail(LBCH_EINVAL, "NULL handle");
     if (hook == LBCH_HOOK_SKIP_FIRST_LOAD) {
         h->debug_skip = value ? 1 : 0;
+        if (value && use_sweep(h)) {  // the sweep has no bounded wait to run out
+            h->force_tile = true;
+            h->shape = 0;
+            drop_graphs(h);
+        }
         return LBCH_OK;
     }
     if (hook == LBCH_HOOK_NO_PDL) {

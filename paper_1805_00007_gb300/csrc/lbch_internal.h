@@ -51,7 +51,7 @@ struct lbch_handle {
     int shape = 0;              // tile shape in use (index into the precision's shape list)
     bool tau1 = false;          // every instance has tau_g = 1: the populations drop out of the step
     bool force_general = false; // test hook: keep the populations even when tau1 holds
-    bool force_tile = false;    // test hook: step with the tile kernel instead of the row sweep
+    bool force_tile = false;    // step with the tile kernel instead of the row sweep
     bool pair = false;          // step two at a time with the two-step kernel (when pair_ok holds); odd
     int pshape = 0;             // steps take the one-step kernel above; pshape indexes pair_shape()
     bool walls = false;         // an instance has walls
