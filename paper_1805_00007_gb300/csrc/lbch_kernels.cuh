@@ -429,7 +429,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned parity)
     return ok != 0;
 }
 
-// Bounded wait: gives up after `limit` polls (each poll may suspend the thread for a short while).
+// Bounded wait: gives up after `limit` polls (each poll may suspend the thread for a short while, 3.7 us as measured: WAIT_POLLS
+// run out after a second, where a copy takes microseconds).
+constexpr unsigned WAIT_POLLS = 1u << 18;
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, unsigned parity, unsigned limit)
 {
     for (unsigned k = 0; k < limit; k++)
@@ -691,13 +693,13 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : (sizeof(C) == 8 ? 2 : 3)) 
         if (t >= a.total_tiles) break;
         const int s = it & 1;
         // every thread observes the completion of the stage's copies itself (bounded wait)
-        bool ok = mbar_wait_bounded(&mbar[s], (unsigned)((it >> 1) & 1), 1u << 22);
+        bool ok = mbar_wait_bounded(&mbar[s], (unsigned)((it >> 1) & 1), WAIT_POLLS);
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {
                 atomicOr(&a.ctl->err, 1u);
                 // let a copy already issued into the other stage land before the CTA exits (bounded)
                 if (t + stride < a.total_tiles)
-                    mbar_wait_bounded(&mbar[s ^ 1], (unsigned)(((it + 1) >> 1) & 1), 1u << 22);
+                    mbar_wait_bounded(&mbar[s ^ 1], (unsigned)(((it + 1) >> 1) & 1), WAIT_POLLS);
             }
             break;  // skip the remaining tiles; the step counter below is still kept consistent
         }

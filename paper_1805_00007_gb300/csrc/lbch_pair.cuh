@@ -505,9 +505,9 @@ __global__ void __launch_bounds__(NT, NT > 512 ? 1 : 2) ch_pair_kernel(const __g
     // error, lets the copy land if it was issued (bounded again) so that no copy into this CTA's shared
     // memory outlives it, and tells the CTA to stop; the step counter is still kept consistent below.
     auto wait_tables = [&]() {
-        if (!mbar_wait_bounded(&s_tbar, (unsigned)(tuse & 1), 1u << 22)) {
+        if (!mbar_wait_bounded(&s_tbar, (unsigned)(tuse & 1), WAIT_POLLS)) {
             atomicOr(&a.ctl->err, 1u);
-            mbar_wait_bounded(&s_tbar, (unsigned)(tuse & 1), 1u << 22);
+            mbar_wait_bounded(&s_tbar, (unsigned)(tuse & 1), WAIT_POLLS);
             s_abort = 1;
         }
         tuse++;
