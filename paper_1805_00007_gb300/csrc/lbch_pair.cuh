@@ -105,7 +105,7 @@ __device__ __forceinline__ void pair_mu_div(const P* ph, const C* sX1, const C* 
 // W, height H; mu and D come from the region one node wider (stride MW), phi from the region two nodes
 // wider (stride PW), the velocity at table index (row, col) + tu.  The nine post-collision populations
 // are stored as planes of W * H values, the axis directions in a quarter (collide9).
-template <typename C, typename P, int W, int H, int MW, int PW, int NT, bool kShift>
+template <typename C, typename P, int W, int H, int MW, int PW, int NT>
 __device__ __forceinline__ void pair_collide(const P* ph_reg, const C* s_mu, const C* s_D, const C* sX1,
                                              const C* sX2, const C* sY1, const C* sY2, int tu, const Consts<C>& K0,
                                              bool model2, C* s_post)
@@ -124,7 +124,7 @@ __device__ __forceinline__ void pair_collide(const P* ph_reg, const C* s_mu, con
         node_flow(ph, ux, uy, K0, Px, Py);
         node_force(ph, gmx, gmy, gDx, gDy, Px, Py, model2, K0, Jx, Jy);
         collide9<C, true>(s_mu[m], ux, uy, Px, Py, Jx, Jy, nullptr, K0, post);
-        if (!kShift) post[0] = rest_add(post[0], ph, K0);
+        post[0] = rest_add(post[0], ph, K0);
 #pragma unroll
         for (int q = 0; q < 9; q++) s_post[q * (W * H) + e] = post[q];
     });
@@ -252,20 +252,14 @@ __device__ __forceinline__ float2 pair_pull2(const float* s_post, int r, int c, 
 }
 
 // phi(t+1) = phi(t) + g_0 + sum_q g_q on the float path: hi + lo absorbs the increment exactly (TwoSum),
-// as in the one-step kernels; on the double path phi(t+1) is the plain sum.
-template <typename C, typename P, bool kFF>
-__device__ __forceinline__ P pair_phi(P h_in, float lo_in, C v0, C sumq, float& lo_out)
+// as in the one-step kernels.  (On the double path phi(t+1) is the plain sum.)
+__device__ __forceinline__ float pair_phi(float h, float lo_in, float v0, float sumq, float& lo_out)
 {
-    if (kFF) {
-        const float h = (float)h_in;
-        const float tt = lo_in + (float)(v0 + sumq);
-        const float sm = h + tt;
-        const float bb = sm - h;
-        lo_out = (h - (sm - bb)) + (tt - bb);
-        return (P)sm;
-    }
-    lo_out = 0.0f;
-    return (P)(v0 + sumq);
+    const float tt = lo_in + (v0 + sumq);
+    const float sm = h + tt;
+    const float bb = sm - h;
+    lo_out = (h - (sm - bb)) + (tt - bb);
+    return sm;
 }
 
 // Shared-memory views of one CTA's regions.
@@ -361,8 +355,6 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
                                            int x0, int y0, int pitch, long long rb, P* phi_out, float* lo_out)
 {
     using L = PairShape<C, P, TX, TY>;
-    constexpr bool kFF = L::FF;
-    constexpr bool kShift = sizeof(C) == 4;  // float arithmetic carries g_0 - phi
     constexpr int W6 = L::W6, W3 = L::W3;
     const Consts<C>& K0 = consts<C>(I);
     const bool model2 = I.model == 2;
@@ -388,7 +380,7 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
         for_images3(gx, gy, nx, ny, 0, [&](int xx, int yy) { phi_out[rb + (long long)yy * pitch + xx] = hi; });
     };
 
-    if constexpr (kFF) {
+    if constexpr (L::FF) {
         // step t: mu, D on tile + 5; collision on tile + 4; streaming to phi(t+1) on tile + 3
         pair_mu_div2<L::W5, L::H5, W6, NT>(S.phi0, S.X1, S.X2, Ya1, Ya2, 0, K0, model2, S.mu, S.D);
         __syncthreads();
@@ -400,7 +392,7 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
             const float* h = S.phi0 + (r + 3) * W6 + c + 3;
             const float2 l = ld2(S.lo0 + r * W3 + c);
             float la, lb;
-            const float ha = pair_phi<C, P, kFF>(h[0], l.x, v0.x, sum.x, la), hb = pair_phi<C, P, kFF>(h[1], l.y, v0.y, sum.y, lb);
+            const float ha = pair_phi(h[0], l.x, v0.x, sum.x, la), hb = pair_phi(h[1], l.y, v0.y, sum.y, lb);
             st2(S.hi1 + r * W3 + c, ha, hb);
             st2(S.lo1 + r * W3 + c, la, lb);
         });
@@ -418,8 +410,8 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
             const float2 sum = pair_pull2<TX, L::N1>(S.post, r, c, v0);
             const int k = (r + 3) * W3 + c + 3;
             float la, lb;
-            const float ha = pair_phi<C, P, kFF>(S.hi1[k], S.lo1[k], v0.x, sum.x, la);
-            const float hb = pair_phi<C, P, kFF>(S.hi1[k + 1], S.lo1[k + 1], v0.y, sum.y, lb);
+            const float ha = pair_phi(S.hi1[k], S.lo1[k], v0.x, sum.x, la);
+            const float hb = pair_phi(S.hi1[k + 1], S.lo1[k + 1], v0.y, sum.y, lb);
             const long long node = rb + (long long)gy * pitch + gx;
             if (gx + 1 < nx) {
                 st2(phi_out + node, ha, hb);
@@ -431,41 +423,31 @@ __device__ __forceinline__ void pair_steps(const PairSmem<C, P, TX, TY>& S, cons
             images(gx, gy, ha);
             if (gx + 1 < nx) images(gx + 1, gy, hb);
         });
-        return;
+    } else {
+        pair_mu_div<C, P, L::W5, L::H5, W6, NT>(S.phi0, S.X1, S.X2, Ya1, Ya2, 0, K0, model2, S.mu, S.D);
+        __syncthreads();
+        pair_collide<C, P, L::W4, L::H4, L::W5, W6, NT>(S.phi0, S.mu, S.D, S.X1, S.X2, Ya1, Ya2, 2, K0, model2, S.post);
+        __syncthreads();
+        for_region<W3, L::H3, NT>([&](int e, int r, int c) {
+            C v0;
+            const C sumq = pair_pull<C, W3, L::N4>(S.post, r, c, v0);
+            S.hi1[e] = v0 + sumq;
+        });
+        __syncthreads();
+        pair_mu_div<C, P, L::W2, L::H2, W3, NT>(S.hi1, S.X1, S.X2, Yb1, Yb2, 3, K0, model2, S.mu, S.D);
+        __syncthreads();
+        pair_collide<C, P, L::W1, L::H1, L::W2, W3, NT>(S.hi1, S.mu, S.D, S.X1, S.X2, Yb1, Yb2, 5, K0, model2, S.post);
+        __syncthreads();
+        for_region<TX, TY, NT>([&](int e, int r, int c) {
+            const int gx = x0 + c, gy = y0 + r;
+            if (gx >= nx || gy >= ny) return;
+            C v0;
+            const C sumq = pair_pull<C, TX, L::N1>(S.post, r, c, v0);
+            const P hi = v0 + sumq;
+            phi_out[rb + (long long)gy * pitch + gx] = hi;
+            images(gx, gy, hi);
+        });
     }
-
-    // step t: mu, D on tile + 5; collision on tile + 4; streaming to phi(t+1) on tile + 3
-    pair_mu_div<C, P, L::W5, L::H5, W6, NT>(S.phi0, S.X1, S.X2, Ya1, Ya2, 0, K0, model2, S.mu, S.D);
-    __syncthreads();
-    pair_collide<C, P, L::W4, L::H4, L::W5, W6, NT, kShift>(S.phi0, S.mu, S.D, S.X1, S.X2, Ya1, Ya2, 2, K0, model2, S.post);
-    __syncthreads();
-    for_region<W3, L::H3, NT>([&](int e, int r, int c) {
-        C v0;
-        const C sumq = pair_pull<C, W3, L::N4>(S.post, r, c, v0);
-        float lo1;
-        S.hi1[e] = pair_phi<C, P, kFF>(S.phi0[(r + 3) * W6 + c + 3], kFF ? S.lo0[e] : 0.0f, v0, sumq, lo1);
-        if (kFF) S.lo1[e] = lo1;
-    });
-    __syncthreads();
-
-    // step t+1: mu, D on tile + 2; collision on tile + 1; streaming to phi(t+2) on the tile
-    pair_mu_div<C, P, L::W2, L::H2, W3, NT>(S.hi1, S.X1, S.X2, Yb1, Yb2, 3, K0, model2, S.mu, S.D);
-    __syncthreads();
-    pair_collide<C, P, L::W1, L::H1, L::W2, W3, NT, kShift>(S.hi1, S.mu, S.D, S.X1, S.X2, Yb1, Yb2, 5, K0, model2, S.post);
-    __syncthreads();
-    for_region<TX, TY, NT>([&](int e, int r, int c) {
-        const int gx = x0 + c, gy = y0 + r;
-        if (gx >= nx || gy >= ny) return;
-        C v0;
-        const C sumq = pair_pull<C, TX, L::N1>(S.post, r, c, v0);
-        const int h1 = (r + 3) * W3 + c + 3;
-        float lo;
-        const P hi = pair_phi<C, P, kFF>(S.hi1[h1], kFF ? S.lo1[h1] : 0.0f, v0, sumq, lo);
-        const long long node = rb + (long long)gy * pitch + gx;
-        phi_out[node] = hi;
-        if (kFF) lo_out[node] = lo;
-        images(gx, gy, hi);
-    });
 }
 
 // The instance and origin of tile t.
