@@ -33,12 +33,11 @@ from paper_1805_00007_gb300 import workloads as wl  # noqa: E402
 REV_N = 256
 METRIC = "MLUPS and % HBM roofline (FP32 vs FP64 step) at stated phi error vs FP64 oracle"
 
-# FP32 operations per lattice update of the row-sweep step at tau_g = 1, Model II, float-float phi, the stencils taken
-# column first and the constants folded (a fused multiply-add counts 2): 34 additions, 17 products and 30 fused
-# multiply-adds per node, from the instruction counts of a launch on 3001 x 1999 over the nodes it forms, halo included.
-FLOPS_PER_LU_TAU1 = 111
-# The FP64 step does the same operations without the TwoSum (6 fewer) and with a reciprocal refined by two
-# Newton steps (6 more): 111 as well.
+# Operations per lattice update of the step at tau_g = 1, Model II, as its source forms them (a fused multiply-add counts 2; the
+# halo that tiles and strips form twice, and the approximation in the force's reciprocal, not counted): in float 37 additions, 17
+# products and 32 fused multiply-adds, the float-float sum of phi included; in double, without it and with the rest
+# population and the reciprocal's third-order step, 30, 17 and 34.
+FLOPS_PER_LU_TAU1 = {"f32": 118, "f64": 115}
 SMS, FP32_LANES_PER_SM, FP64_LANES_PER_SM = 152, 128, 2
 
 # Algorithmic HBM bytes per lattice update of the general step (any tau_g): the nine populations read and
@@ -306,7 +305,7 @@ def run_case(case, nsteps, tile=0, form="sweep"):
                 abi.lb_ch_adjoint_step(sim.h, tape.data_ptr(), 4 + nsteps - 1 - k)
             torch.cuda.synchronize()
         print(json.dumps({"case": case, "adjoint_steps": nsteps,
-                          "kernels": "adj::fwd_mu, adj::local, adj::transpose1, adj::transpose2"}))
+                          "kernels": "adj::local, adj::transpose"}))
         return
     if parts[0] == "ens":  # the first N instances of the ragged shear ensemble, e.g. ens_f32_64 or ens_f32_64_0.8
         from paper_1805_00007_gb300 import workloads as wl
@@ -723,8 +722,8 @@ def main():
     sm_mhz = (clocks or {}).get("sm_mhz") or 2070.0
     peak_tflops = SMS * FP32_LANES_PER_SM * 2 * sm_mhz * 1e6 / 1e12
     peak64_tflops = SMS * FP64_LANES_PER_SM * 2 * sm_mhz * 1e6 / 1e12
-    alu_tflops = FLOPS_PER_LU_TAU1 * nodes * spl32 / launch32 / 1e12
-    alu64_tflops = FLOPS_PER_LU_TAU1 * nodes / (t64 / rev) / 1e12
+    alu_tflops = FLOPS_PER_LU_TAU1["f32"] * nodes * spl32 / launch32 / 1e12
+    alu64_tflops = FLOPS_PER_LU_TAU1["f64"] * nodes / (t64 / rev) / 1e12
     # the FMA throughput the device sustains (lb_ch_alu_peak), beside the unit-count peaks
     fma32 = abi.lb_ch_alu_peak(abi.LBCH_F32, stream.cuda_stream) / 1e12
     fma64 = abi.lb_ch_alu_peak(abi.LBCH_F64, stream.cuda_stream) / 1e12
@@ -746,7 +745,7 @@ def main():
                      "revolution_ms": {"best": 1e3 * min(times64), "median": 1e3 * statistics.median(times64),
                                        "n": len(times64)},
                      "achieved_gbs": achieved64, "frac": achieved64 / hbm_peak, "kernel": kernel_name(kern64, "f64"),
-                     "alu": {"flops_per_lu": FLOPS_PER_LU_TAU1, "achieved": alu64_tflops, "peak": peak64_tflops,
+                     "alu": {"flops_per_lu": FLOPS_PER_LU_TAU1["f64"], "achieved": alu64_tflops, "peak": peak64_tflops,
                              "unit": "TFLOP/s", "frac": alu64_tflops / peak64_tflops,
                              "peak_from": "152 SMs x 2 FP64 lanes x 2 flop x median SM clock under load",
                              "peak_measured": fma64, "frac_of_measured": alu64_tflops / fma64}},
@@ -760,7 +759,7 @@ def main():
                                            "written once per launch of two steps"},
                          "l2_resident": "one 256^2 field is 0.5 MB: the state stays in L2, so HBM does not bound it",
                          "peak_kind": peak_kind, "us_per_launch": launch32 * 1e6,
-                         "alu": {"flops_per_lu": FLOPS_PER_LU_TAU1, "achieved": alu_tflops, "peak": peak_tflops,
+                         "alu": {"flops_per_lu": FLOPS_PER_LU_TAU1["f32"], "achieved": alu_tflops, "peak": peak_tflops,
                                  "unit": "TFLOP/s", "frac": alu_tflops / peak_tflops,
                                  "peak_from": "152 SMs x 128 FP32 lanes x 2 flop x median SM clock under load",
                                  "peak_measured": fma32, "frac_of_measured": alu_tflops / fma32}},

@@ -104,7 +104,7 @@ typedef struct {
     int model;           /* 1: Model I; 2: Model II (Eq. mark3 force added); 3: Model II with the complete
                             diffusive-scale force of Eq. F2-1, whose time derivatives are backward
                             differences over one step (zero at step 0); steps with the row sweep's
-                            Model III build (its two unrolled configurations) or the tile kernel, not
+                            Model III build (its first two configurations) or the tile kernel, not
                             with the adjoint, the coupled flow or slabs */
     int vel;             /* lbch_vel */
     int nvort;           /* vortex count of the deformation field */

@@ -721,8 +721,8 @@ void stage_give(double* p, size_t bytes)
 
 // Warps per block for n strips: on a grid that fills the device, blocks as large as an SM takes keep the SM's warps on
 // neighbouring strips of the same rows, and so on few pages and DRAM rows (4096^2, us per step in blocks of 2, 8 and 16
-// warps: half storage with the populations 187, 184, 175; float at tau_g = 1 119, 118, 116); smaller grids want their
-// strips on as many SMs as there are (100^2: 3.4 us in blocks of two, 5.2 in blocks of 16).
+// warps: half storage with the populations 147, 142, 136; float 253, 249, 248, at tau_g = 1 87.2, 86.5, 85.7); smaller
+// grids want their strips on as many SMs as there are (100^2: 3.5 us in blocks of two, 4.7 in blocks of 16).
 int sweep_block(const SweepFit& fit, long long n)
 {
     int nw = 2;
@@ -1136,17 +1136,17 @@ void choose_default(lbch_handle* h, int sms)
     const bool tau1 = h->tau1;
     // the row sweep: on grids so small that sixteen warps per SM would get two rows each or fewer (in float at tau_g = 1 five,
     // a row being shorter there), strips for half as many warps (eight in double: a quarter) step faster: at tau_g = 1 in
-    // float 448^2 4.9 against 5.6, 768^2 7.5 against 7.9, 900^2 8.8 against 8.7; with the populations 384^2 7.5 against
-    // 8.0, 600^2 10.7 against 10.1; double 256^2 36 against 54
+    // float 448^2 4.9 against 5.5, 768^2 7.6 against 7.8, 900^2 8.8 against 8.6; with the populations 384^2 7.0 against
+    // 7.4, 600^2 9.7 against 9.9; double 256^2 36 against 54
     const lbch_handle::SweepCut& cut = h->sw[0][sweep_gen(h)];
     h->shape = h->prec == LBCH_F64 ? (cut.rows_per <= 8 && !h->model3 ? 2 : 0) : (cut.rows_per <= (h->prec == LBCH_F32 && tau1 ? 5 : 2) ? 1 : 0);
     if (h->model3) return;
     auto tiles = [&](int k) { return h->ps[k].total_tiles; };
     if (h->prec == LBCH_F64) {
-        // The tile kernel while its waves are few, where strips would be short (500^2: 59 against 69); the row sweep on
-        // grids of a dozen waves (1024^2 at tau_g = 1: 223 against 229; 724^2: 121 against 115).  Small grids take the
-        // smallest tiles that leave no SM two of them (100^2: 7.8 against 16.0 with 32 x 14), others the shape of
-        // the least waves times the time of one (32 x 16: 16.7 at tau_g = 1, 32 x 14: 14.9).
+        // The tile kernel while its waves are few, where strips would be short (500^2: 59 against 68); the row sweep on
+        // grids of a dozen waves (1024^2 at tau_g = 1: 222 against 229; 724^2: 118 against 115).  Small grids take the
+        // smallest tiles that leave no SM two of them (100^2: 7.5 against 15.6 with 32 x 14), others the shape of
+        // the least waves times the time of one (167 to 149; 256^2, one wave of 32 x 16 and of 32 x 14: 17.6 and 15.8).
         if (tiles(3) > 12 * sms) return;
         h->force_tile = true;
         auto waves = [&](int k) { return (tiles(k) + sms - 1) / sms; };
@@ -1155,19 +1155,19 @@ void choose_default(lbch_handle* h, int sms)
     }
     if (h->prec == LBCH_F16S && tau1) return;  // the tile kernel would round the populations to half
     if (!tau1) {
-        // with the populations: small tiles on small grids (100^2: 2.9 against the sweep's 4.5; 200^2: 4.1), one wave of
-        // 32 x 16 (256^2: 4.5 against 6.0), 32 x 8 up to three per SM (300^2: 5.7 against 6.1), then the row sweep
-        // (384^2: 7.5 against 7.9)
+        // with the populations: small tiles on small grids (100^2: 2.9 against the sweep's 4.5; 200^2: 4.0 against 4.8), one
+        // wave of 32 x 16 (256^2: 4.5 against 5.9), 32 x 8 up to three per SM (300^2: 5.7 against 6.0), then the row sweep
+        // (384^2: 7.0 against 7.2)
         if (2 * tiles(2) <= 5 * sms) { h->force_tile = true; h->shape = 2; }
         else if (tiles(3) <= sms) { h->force_tile = true; h->shape = 3; }
         else if (tiles(1) <= 3 * sms) { h->force_tile = true; h->shape = 1; }
         return;
     }
     // tau_g = 1 in float: the two-step kernel on periodic grids up to two and a half of its 32 x 14 tiles per SM -- 16 x 8
-    // and 32 x 8 tiles while every SM gets one (100^2: 1.5 per step against the row sweep's 3.7; 160^2: 1.8), 32 x 14 up to
-    // two (256^2: 2.0 against 4.3; 320^2: 3.1 against 4.4), 32 x 16 up to two (384^2: 3.6 against 5.1), 32 x 14 from there
-    // (400^2: 4.7 against 5.0) --, otherwise the row sweep (448^2: 4.9 against 5.9).  The odd last step of a call, and taped steps, take
-    // the one-step kernel that is faster there: 16 x 8 tiles up to three per SM (100^2: 2.7 against 4.0).
+    // and 32 x 8 tiles while every SM gets one (100^2: 1.5 per step against the row sweep's 3.5; 160^2: 1.7 against 3.4), 32 x 14 up to
+    // two (256^2: 2.0 against 4.2; 320^2: 3.0 against 4.4), 32 x 16 up to two (384^2: 3.5 against 4.9), 32 x 14 from there
+    // (400^2: 4.66 against 4.71) --, otherwise the row sweep (448^2: 4.8 against 5.8).  The odd last step of a call, and taped steps, take
+    // the one-step kernel that is faster there: 16 x 8 tiles up to three per SM (100^2: 2.6 against 3.5).
     if (!pair_ok(h)) return;
     auto pairs = [&](int k) { return h->pr[k].total_tiles; };
     h->pair = true;
@@ -1610,7 +1610,7 @@ lbch_status lb_ch_info(lbch_handle* h, double* out)
         bytes = 2.0 * ((double)h->phi_elem + (h->lo[0] ? 4.0 : 0.0));
     if (use_pair(h)) bytes *= 0.5;     // the two-step kernel reads and writes phi once per two updates
     if (h->model3) bytes += 2.0 * 2.0 * (double)h->c_elem();  // H of Model III, read and written
-    if (h->coupled) {  // f and g read and written, phi read and written, u and p written and read
+    if (h->coupled) {  // f and g read and written, phi read and written, u and p written and read (mu can be formed again from phi)
         const double e = h->prec == LBCH_F64 ? 8.0 : 4.0;
         bytes = 2.0 * (18.0 * e + e) + 2.0 * 3.0 * e;
     }

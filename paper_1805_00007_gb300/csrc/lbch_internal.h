@@ -12,7 +12,7 @@ struct Shape { int tx, ty, nt; };  // output nodes of a tile, threads per block
 
 // Configurations of the row-sweep kernel: the warps per SM among which the grid is cut into strips (fewer where the
 // kernel's registers allow fewer).  Many warps hide latency and give long runs of rows on large grids; a grid whose
-// strips would get only a few rows each steps faster with fewer, longer ones (lb_ch_tune; sweep_cost).  A
+// strips would get only a few rows each steps faster with fewer, longer ones (choose_default, lb_ch_tune).  A
 // configuration is reported under a nominal tile of 56 columns.
 constexpr int kSweepShapes = 4;
 constexpr int kM3SweepShapes = 2;  // configurations used for handles with a Model III instance
@@ -20,8 +20,8 @@ constexpr int kSweepWarps[kSweepShapes] = {16, 8, 4, 12};
 constexpr int kSweepTileRows[kSweepShapes] = {48, 24, 12, 24};
 constexpr int kSweepW = 56;
 inline Shape sweep_tile(int k) { return Shape{kSweepW, kSweepTileRows[k], 0}; }
-// What a sweep kernel allows on the device: warps resident per SM, SMs, and the columns of its strips.
-// (and of one block).
+// What a sweep kernel allows on the device: warps resident per SM, SMs, warps of one block at most, the output columns of a
+// strip, and the domain columns that the first strip starts before column 0.
 struct SweepFit { int warps, sms, nw, width, lead; };
 
 // Tile shapes of the two-step kernel (periodic instances, tau_g = 1; f32 and f64 only).

@@ -175,8 +175,9 @@ __device__ __forceinline__ int mirror(int j, int n)
 // The isotropic nine-point stencils are products of one-dimensional ones, and are evaluated as such: first a few
 // values per column from the nodes below, at and above a row, then their combination along the row.  A form
 // that holds the column values (the row sweep) forms them once per node, and every constant that another can
-// carry is folded into it at set-up.  A node's update at tau_g = 1, Model II, takes 87 operations this way
-// (streaming and the float-float sum included) where the nine-point forms direction by direction took 149.  The
+// carry is folded into it at set-up.  A node's update at tau_g = 1, Model II, takes 86 operations this way
+// in float (37 additions, 17 products, 32 fused multiply-adds, streaming and the float-float sum included) and 81 in double (30, 17
+// and 34), and the reciprocal's approximation, where the nine-point forms direction by direction took 149.  The
 // FP64 kernels, which the FP64 pipe bounds, and the row sweeps, which instruction issue bounds, gained most
 // (us per step before -> after: FP64 500^2 row sweep 147 -> 94, FP64 256^2 two-step kernel 30.6 -> 23.8, float
 // 3001 x 1999 row sweep 65.7 -> 53.3, half storage with the populations at 4096^2 267 -> 219; float with the

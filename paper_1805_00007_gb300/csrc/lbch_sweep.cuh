@@ -18,20 +18,21 @@
 // node and cross one lane boundary as one number, as do 3, 6, 7 from the right (the grouping of the sum is the one
 // the tile kernel uses too).
 //
-// GEN (any tau_g): the populations are read and written as well.  The warp copies them into a four-slot ring of rows in
-// shared memory (cp.async), three rows ahead of their collision, and phi and its low part two rows ahead.  After the collision the nine g* of a node reach their destinations individually --
-// 1, 5, 8 from the lane to the left, 3, 6, 7 from the right, 2 and 4 from the rows below and above -- and g(t+1) is
-// stored plane by plane.
+// GEN (any tau_g): the populations are read and written as well.  The warp copies what a step takes -- the populations of
+// its collision row, its row of phi, the low part of its output row -- into a ring of slots in shared memory (cp.async), one
+// step ahead in float, two in double and half storage (SweepShape::AHEAD; twice as many slots).  After the collision the
+// nine g* of a node reach their destinations individually -- 1, 5, 8 from the lane to the left, 3, 6, 7 from the right,
+// 2 and 4 from the rows below and above -- and g(t+1) is stored plane by plane.
 //
 // Division of work.  Every warp is on its own: it loads its rows of phi straight into registers, two rows ahead,
 // and no block-wide wait joins it to others, so the length of its strip is free and the host cuts the grid to the
 // device -- as many strips as the warps it wants resident, all of one length (sweep_rows).  A strip of R rows
 // computes mu on R + 4 rows and collides R + 2: on a large grid R is near a hundred, where tiles of twelve rows per
 // warp staged through shared memory computed a third of their mu and a seventh of their collisions twice.  Measured
-// against that form (us per step, one GB300): 4096^2 tau_g = 0.8 in float 295 -> 249 (5.9 TB/s of 88 B per update: bound
-// by HBM), half storage 219 -> 175; tau_g = 1 in float 3001 x 1999 53 -> 49, 512^2 10.4 -> 6.2, 100^2 4.0 (was 10.4), an
-// ensemble of 48 instances with walls 68 -> 35 (instruction issue, 70 % busy at 150 instructions per update, of which
-// 100 are the arithmetic).
+// against that form (us per step, one GB300; now with the image stores below): 4096^2 tau_g = 0.8 in float 295 -> 248 (5.95
+// TB/s of 88 B per update: bound by HBM), half storage 219 -> 136; tau_g = 1 in float 3001 x 1999 53 -> 32.7, 512^2
+// 10.4 -> 6.1, 100^2 10.4 -> 3.5, an ensemble of 48 instances with walls 68 -> 26.6 (instruction issue, 77 % busy while an SM
+// has work, at 159 instructions per update, of which 102 are the arithmetic).
 #pragma once
 #include <type_traits>
 
@@ -83,8 +84,8 @@ struct SweepShape {
     static constexpr int LEAD = GEN ? 0 : 1;           // domain columns the first strip starts before column 0
     static constexpr int NQ = sizeof(S) == 2 ? 8 : 9;  // stored population planes
     // Rows under way per warp.  In float the step is bound by HBM, which serves 16 warps per SM best with one row each
-    // under way (4096^2, us per step: 249 with one, 302 with two, 318 with three); the others hide latency with two (half
-    // storage: 175 and 172).
+    // under way (4096^2, us per step: 248 with one, 269 with two); the others hide latency with two (half storage: 153 with
+    // one, 136 with two).
     static constexpr int AHEAD = FF ? 1 : 2;
     static constexpr int RING = 2 * AHEAD;             // ring slots per warp: a power of two above AHEAD
     static constexpr size_t SLOT = (size_t)NQ * BW * sizeof(S) + BW * sizeof(P) + (FF ? BW * 4 : 0);
