@@ -702,7 +702,7 @@ cudaError_t stage_take(size_t bytes, double** p, size_t* got)
     return cudaSuccess;
 }
 
-// back to the cache, or freed when the cache is full (the smallest kept buffer makes room for a larger one)
+// back to the cache, or freed when the cache is full
 void stage_give(double* p, size_t bytes)
 {
     if (!p) return;

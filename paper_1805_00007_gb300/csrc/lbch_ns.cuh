@@ -21,8 +21,8 @@
 // stencil operand at a ghost row beyond a wall takes the value of the mirror node: a staged operand is read at that node,
 // and a derived one is formed at the mirror row of the tile's region.
 //
-// What bounds it: in float the instructions issued (about 390 and 600 per node) and, on small grids, the latency of two
-// launches (3 us each); in double the FP64 pipe.  256 x 1024 in float: 14.5 us per step, against 17.9 with a plane per
+// What bounds it: in float the instructions issued (387 and 662 per node) and, on small grids, the latency of two
+// launches (3 us each); in double the FP64 pipe.  256 x 1024 in float: 14.3 us per step, against 17.9 with a plane per
 // population, ordinary launches and the populations g read at tau_g = 1 too; 64 x 200: 5.9 against 11.1.  One thread per
 // node against two nodes per thread in the collision: 5.9 and 7.1 us for 64 x 200, 11.8 and 14.4 for 200 x 760, 20.2 and
 // 19.8 for 400 x 1000, and in double 101 and 155 for 160 x 640.
