@@ -15,6 +15,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -442,7 +443,8 @@ cudaError_t launch_step(lbch_handle* h, int parity)
 cudaError_t time_table(lbch_handle* h, int steps)
 {
     if (!h->timed) return cudaSuccess;
-    time_table_kernel<<<time_table_blocks(steps, h->n_inst), TIME_NT, 0, h->stream>>>(h->d_inst, h->n_inst, h->ctl, steps, h->d_T);
+    const auto kernel = (long long)steps * h->n_inst <= INT_MAX - TIME_NT ? time_table_kernel<int> : time_table_kernel<long long>;
+    kernel<<<time_table_blocks(steps, h->n_inst), TIME_NT, 0, h->stream>>>(h->d_inst, h->n_inst, h->ctl, steps, h->d_T);
     return cudaGetLastError();
 }
 
