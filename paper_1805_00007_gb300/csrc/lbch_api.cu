@@ -1301,7 +1301,8 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     CKI(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     if (!coupled) {
         CKI(cut_sweeps(h, !h->tau1));
-        for (int sk = 0; sk < kPairShapes && prec != LBCH_F16S; sk++) {
+        // (the two-step kernel for those handles that it can step: its four tables take some 45 us)
+        for (int sk = 0; sk < kPairShapes && pair_ok(h); sk++) {
             CKI(lbch_prepare_pair(h, sk));
             CKI(dalloc(h, &h->pr[sk].d_tile_begin, sizeof(int) * (n_inst + 1)));
             CKI(cudaMemcpyAsync(h->pr[sk].d_tile_begin, pair_begin[sk].data(), sizeof(int) * (n_inst + 1),
