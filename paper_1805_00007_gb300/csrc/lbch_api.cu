@@ -1301,8 +1301,7 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     CKI(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     if (!coupled) {
         CKI(cut_sweeps(h, !h->tau1));
-        // (the two-step kernel for those handles that it can step: its four tables take some 45 us)
-        for (int sk = 0; sk < kPairShapes && pair_ok(h); sk++) {
+        for (int sk = 0; sk < kPairShapes && prec != LBCH_F16S; sk++) {
             CKI(lbch_prepare_pair(h, sk));
             CKI(dalloc(h, &h->pr[sk].d_tile_begin, sizeof(int) * (n_inst + 1)));
             CKI(cudaMemcpyAsync(h->pr[sk].d_tile_begin, pair_begin[sk].data(), sizeof(int) * (n_inst + 1),
@@ -1364,7 +1363,8 @@ lbch_status init_impl(const lbch_params* params, int n_inst, const double* phi0,
     CKI(cudaMemcpyAsync(h->d_node_begin, h->node_begin.data(), sizeof(long long) * (n_inst + 1), cudaMemcpyHostToDevice, h->stream));
     CKI(cudaMemcpyAsync(h->d_tabs, tabs.data(), sizeof(double) * tabs.size(), cudaMemcpyHostToDevice, h->stream));
     CKI(cudaMemcpyAsync(h->d_tabs_f, tabs_f.data(), sizeof(float) * tabs_f.size(), cudaMemcpyHostToDevice, h->stream));
-    for (int sk = 0; sk < kPairShapes && h->pr[sk].d_ttabs; sk++) CKI(lbch_pair_tables(h, sk));
+    // (the two-step kernel's tables where it can step the handle: the four launches take some 20 us)
+    for (int sk = 0; sk < kPairShapes && pair_ok(h); sk++) CKI(lbch_pair_tables(h, sk));
     CKI(cudaMemsetAsync(h->ctl, 0, sizeof(Ctl), h->stream));
     for (int k = 0; k < 2; k++) {
         CKI(cudaMemsetAsync(h->g[k], 0, gbytes, h->stream));
